@@ -135,6 +135,16 @@ Engine::~Engine() {
     if (fork_ev_[o]) cudaEventDestroy(fork_ev_[o]);
 }
 
+void Engine::set_taps() {
+  S_ = P_.n_scales;
+  for (int m = 0; m < 2; m++) base_R_[m] = gaussian_taps(base_sigma(P_, m == 1), &base_t_[m]);
+  for (int i = 1; i <= S_ + 2; i++) {
+    const double k = std::sqrt(level_sigma(P_, i) * level_sigma(P_, i) -
+                               level_sigma(P_, i - 1) * level_sigma(P_, i - 1));
+    lvl_R_[i] = gaussian_taps(k, &lvl_t_[i]);
+  }
+}
+
 sift_status Engine::init() {
   if (inited_) return SIFT_OK;
   std::string why;
@@ -144,7 +154,6 @@ sift_status Engine::init() {
   }
   cudaError_t e = cudaGetDevice(&dev_);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm_, cudaDevAttrMultiProcessorCount, dev_);
-  if (e == cudaSuccess) e = blur_set_attributes();
   if (e == cudaSuccess) e = descriptor_set_attributes();
   if (e == cudaSuccess) e = extrema_set_attributes();
   if (e == cudaSuccess) e = cudaMalloc(&ddesc_, sizeof(Desc));
@@ -161,16 +170,14 @@ sift_status Engine::init() {
   }
   for (int o = 0; o < kMaxOct && e == cudaSuccess; o++)
     e = cudaEventCreateWithFlags(&fork_ev_[o], cudaEventDisableTiming);
+  unsigned radii = 0;
+  set_taps();
+  for (int R : base_R_) radii |= 1u << std::max(R, 0);
+  for (int l = 1; l <= S_ + 2; l++) radii |= 1u << lvl_R_[l];
+  if (e == cudaSuccess) e = blur_set_attributes(radii);
   if (e != cudaSuccess) {
     err = std::string("CUDA initialisation failed: ") + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? SIFT_E_OOM : SIFT_E_CUDA;
-  }
-  S_ = P_.n_scales;
-  for (int m = 0; m < 2; m++) base_R_[m] = gaussian_taps(base_sigma(P_, m == 1), &base_t_[m]);
-  for (int i = 1; i <= S_ + 2; i++) {
-    const double k = std::sqrt(level_sigma(P_, i) * level_sigma(P_, i) -
-                               level_sigma(P_, i - 1) * level_sigma(P_, i - 1));
-    lvl_R_[i] = gaussian_taps(k, &lvl_t_[i]);
   }
   tun_ = default_tuning();
   lookback_config(&lb_spins_, &lb_hold_);
@@ -196,13 +203,7 @@ sift_status Engine::init_noalloc() {
     err = std::string("CUDA device query failed: ") + cudaGetErrorString(e);
     return SIFT_E_CUDA;
   }
-  S_ = P_.n_scales;
-  for (int m = 0; m < 2; m++) base_R_[m] = gaussian_taps(base_sigma(P_, m == 1), &base_t_[m]);
-  for (int i = 1; i <= S_ + 2; i++) {
-    const double k = std::sqrt(level_sigma(P_, i) * level_sigma(P_, i) -
-                               level_sigma(P_, i - 1) * level_sigma(P_, i - 1));
-    lvl_R_[i] = gaussian_taps(k, &lvl_t_[i]);
-  }
+  set_taps();
   tun_ = default_tuning();
   lookback_config(&lb_spins_, &lb_hold_);
   ext_max_ = extrema_max_ctas(S_);
@@ -246,7 +247,6 @@ int cand_capacity(long long octave_px) {
   c = std::min<long long>(c, 1 << 22);
   return (int)((c + kChunk - 1) / kChunk * kChunk);
 }
-int tile_h_of(int kind) { return kind == TK_BLUR16 ? 16 : kind == TK_BLUR64 ? 64 : 32; }
 }  // namespace
 
 size_t Engine::workspace_bytes(int n, const int *H, const int *W) const {
@@ -361,21 +361,22 @@ sift_status Engine::fill_plan(int n, const ImgIn *in, Desc &hd, WsLayout &L, int
         if (o < hd.img[b].n_oct) {
           const OctDev &od = hd.oct[hd.img[b].oct0 + o];
           if (k == TK_EXT) t = od.wpr * div_up(od.H, kExtTH);
-          else t = div_up(od.W, kBlurTW) * div_up(od.H, tile_h_of(k));
+          else t = div_up(od.W, kBlurTW) * div_up(od.H, blur_tile_rows(k));
         }
         pre[b + 1] = pre[b] + t;
       }
     }
   }
-  // Base-blur tile queues: octave-0 tiles of the images of each mode (the
-  // other mode's images contribute none).
+  // Base-blur queues: octave-0 tiles of the images of each mode (the other
+  // mode's images contribute none).
   for (int m = 0; m < 2; m++) {
+    const int rows = m == 0 && base_R_[0] > 0 ? blur_tile_rows(TK_BLUR32) : kBaseTileRows;
     int *pre = hd.base_pre[m];
     pre[0] = 0;
-    for (int b = 0; b < n; b++)
-      pre[b + 1] = pre[b] + (hd.img[b].up == m ? hd.tile_pre[TK_BLUR32][0][b + 1] -
-                                                     hd.tile_pre[TK_BLUR32][0][b]
-                                               : 0);
+    for (int b = 0; b < n; b++) {
+      const OctDev &od = hd.oct[hd.img[b].oct0];
+      pre[b + 1] = pre[b] + (hd.img[b].up == m ? div_up(od.W, kBlurTW) * div_up(od.H, rows) : 0);
+    }
   }
   hd.bmc_pre[0] = 0;
   hd.cc_pre[0] = 0;
@@ -460,8 +461,12 @@ sift_status Engine::upload(Desc *hd, size_t bytes, cudaStream_t s) {
   return SIFT_OK;
 }
 
-int Engine::grid_blur(int R, int kind, int mode, int ctas) const {
-  return grid_of(blur_blocks_per_sm(R, kind, mode), ctas);
+int Engine::grid_blur(int R, int kind, int mode, int ctas, int storage) const {
+  return grid_of(blur_blocks_per_sm(R, kind, mode, storage), ctas);
+}
+
+int Engine::level_grid(int o, int l, int kind) const {
+  return grid_blur(lvl_R_[l], kind, o > 0 && l == 1 ? 3 : 0, tun_.blur_ctas[o], storage(o, l));
 }
 
 cudaError_t Engine::enqueue_pyramid(cudaStream_t s, int M, int modes, std::vector<ProfRec> *prof) {
@@ -487,7 +492,7 @@ cudaError_t Engine::enqueue_pyramid(cudaStream_t s, int M, int modes, std::vecto
       for (int m = 1; m >= 0; m--) {
         if (!(modes >> m & 1)) continue;
         rec(PC_BASE, [&] {
-          return launch_base_blur(d, base_R_[m], base_t_[m], TK_BLUR32, m == 1,
+          return launch_base_blur(d, base_R_[m], base_t_[m], m == 1,
                                   grid_blur(base_R_[m], TK_BLUR32, m == 1 ? 2 : 1), s);
         });
       }
@@ -497,7 +502,7 @@ cudaError_t Engine::enqueue_pyramid(cudaStream_t s, int M, int modes, std::vecto
     for (int l = 1; l <= S_ + 2; l++) {
       const int kind = storage(o, l) ? TK_BLUR32 : tun_.lvl_kind[o][l];
       rec(PC_BLUR, [&] {
-        return launch_level_blur(d, o, l, lvl_R_[l], lvl_t_[l], kind, grid_blur(lvl_R_[l], kind, 0, tun_.blur_ctas[o]), s,
+        return launch_level_blur(d, o, l, lvl_R_[l], lvl_t_[l], kind, level_grid(o, l, kind), s,
                                  o > 0 && l == 1, true, storage(o, l));
       });
     }
@@ -540,7 +545,7 @@ cudaError_t Engine::enqueue_all(cudaStream_t s, int M, int modes, std::vector<Pr
       for (int m = 1; m >= 0; m--) {
         if (!(modes >> m & 1)) continue;
         rec(PC_BASE, [&] {
-          return launch_base_blur(d, base_R_[m], base_t_[m], TK_BLUR32, m == 1,
+          return launch_base_blur(d, base_R_[m], base_t_[m], m == 1,
                                   grid_blur(base_R_[m], TK_BLUR32, m == 1 ? 2 : 1), s);
         });
       }
@@ -559,7 +564,7 @@ cudaError_t Engine::enqueue_all(cudaStream_t s, int M, int modes, std::vector<Pr
         if (e == cudaSuccess) e = cudaStreamWaitEvent(side, fork_ev_[o], 0);
       }
       rec_on(on_side ? side : s, PC_BLUR, [&] {
-        return launch_level_blur(d, o, l, lvl_R_[l], lvl_t_[l], kind, grid_blur(lvl_R_[l], kind, 0, tun_.blur_ctas[o]),
+        return launch_level_blur(d, o, l, lvl_R_[l], lvl_t_[l], kind, level_grid(o, l, kind),
                                  on_side ? side : s, o > 0 && l == 1, !(on_side && l == S_ + 1),
                                  storage(o, l));
       });

@@ -30,8 +30,9 @@ enum ProfClass { PC_BLUR = 0, PC_BASE = 1, PC_EXTREMA = 2, PC_DECIMATE = 3, PC_K
 // Launch shapes the autotuner chooses. None of them changes an output bit:
 // tiles and grids only decide which CTA computes what.
 struct Tuning {
-  // Tile-height class (TK_BLUR32 / TK_BLUR64) of the blur that writes level l
-  // of octave o; binary16 levels always take 32-row tiles.
+  // Row class (TK_BLUR32 / TK_BLUR64, the smaller and the larger tile) of the
+  // blur that writes level l of octave o; binary16 levels always take the
+  // smaller one.
   int lvl_kind[kMaxOct][kMaxLevels];
   // Resident CTAs per SM of the persistent grids, 0 meaning the occupancy
   // maximum (larger values are capped by it): the level blurs of octave o, the
@@ -147,6 +148,7 @@ class Engine {
   bool last_extract = false;  // the last run was an extraction (outputs described)
 
  private:
+  void set_taps();  // radii and taps of the base and level blurs
   sift_status fill_plan(int n, const ImgIn *imgs, Desc &hd, WsLayout &lay, int *max_oct) const;
   sift_status ensure_workspace(size_t bytes, cudaStream_t s);
   sift_status upload(Desc *hd, size_t bytes, cudaStream_t s);
@@ -158,7 +160,9 @@ class Engine {
                           bool fork = false);
   sift_status get_graph(int max_oct, int modes, cudaGraphExec_t *out);
   void drop_graphs();
-  int grid_blur(int R, int kind, int mode, int ctas = 0) const;
+  int grid_blur(int R, int kind, int mode, int ctas = 0, int storage = 0) const;
+  // Grid of the launch that writes level l of octave o in row class `kind`.
+  int level_grid(int o, int l, int kind) const;
  public:
   // Grid of the single-pass compactions (their scan runs over blocks).
   int compact_grid() const { return grid_of(cmp_max_, tun_.cmp_ctas); }

@@ -35,8 +35,10 @@ constexpr int kBmCols = 30;        // columns per bitmap word = extrema strip wi
 constexpr int kExtTH = 32;         // extrema tile rows (one warp streams down them)
 constexpr int kChunk = 2048;       // compaction chunk (words or slots)
 
-// Tile-queue kinds: blur with tile height 16/32/64, extrema tiles, decimation.
-enum TileKind { TK_BLUR16 = 0, TK_BLUR32 = 1, TK_BLUR64 = 2, TK_EXT = 3, TK_COUNT = 4 };
+// Work queues: blur tiles of the smaller and the larger row class (blur.cuh; 32
+// and 64 in the tuning's JSON form), extrema tiles.
+enum TileKind { TK_BLUR32 = 0, TK_BLUR64 = 1, TK_EXT = 2, TK_COUNT = 3 };
+constexpr int kBaseTileRows = 32;  // tile rows of the base kernels that work by tiles
 
 // Rejection codes of the refinement (0 = kept).
 enum RefCode { RC_KEEP = 0, RC_SINGULAR = 1, RC_NOCONV = 2, RC_BOUNDS = 3, RC_CONTRAST = 4, RC_EDGE = 5 };
@@ -119,7 +121,8 @@ struct Desc {
   int *fin_flat;               // [kMaxImg + 1] prefix of n_fin over images
   // geometry
   int tile_pre[TK_COUNT][kMaxOct][kMaxImg + 1];
-  int base_pre[2][kMaxImg + 1];  // base-blur tiles (32 rows) of the images with up = 0 / 1
+  // Base-blur work of the images with up = 0 (steps, or tiles at radius 0) / 1 (tiles).
+  int base_pre[2][kMaxImg + 1];
   int bmc_pre[kMaxImg + 1];
   int cc_pre[kMaxImg + 1];
   ImgDev img[kMaxImg];
@@ -205,22 +208,25 @@ __device__ __forceinline__ int refl101(int i, int n) {
 
 // ---------------------------------------------------------------- launchers
 // Pyramid (pyramid.cu)
-cudaError_t launch_base_blur(const Desc *d, int R, const BlurTaps &t, int th_kind, bool upsample,
-                             int grid, cudaStream_t s);
+cudaError_t launch_base_blur(const Desc *d, int R, const BlurTaps &t, bool upsample, int grid,
+                             cudaStream_t s);
 // pdl: launch as a programmatic dependent of the previous kernel on s.
 // storage: 0 FP32 in and out; 1 FP32 source, binary16 output (first level of
 // octave 1 in the fp16 storage mode, from_prev_octave only); 2 binary16 in and
-// out. Binary16 octaves use 32-row tiles.
+// out. Binary16 octaves use the smaller tile.
 cudaError_t launch_level_blur(const Desc *d, int oct, int lvl_out, int R, const BlurTaps &t,
-                              int th_kind, int grid, cudaStream_t s, bool from_prev_octave = false,
-                              bool pdl = true, int storage = 0);
+                              int th_kind, int grid, cudaStream_t s,
+                              bool from_prev_octave = false, bool pdl = true, int storage = 0);
 // Copy one pyramid level (src: the level's first element, `half` for binary16)
 // into a dense H x W FP32 plane.
 cudaError_t launch_export_level(const float *src, bool half, int pitch, int H, int W, float *dst,
                                 cudaStream_t s);
-int blur_smem_bytes(int R, int th_kind);
-int blur_blocks_per_sm(int R, int th_kind, int mode);
-cudaError_t blur_set_attributes();
+// Rows of a tile of a row class.
+int blur_tile_rows(int th_kind);
+// mode: 0 level, 1 base as is, 2 magnified base, 3 level 1 from the previous octave.
+int blur_blocks_per_sm(int R, int th_kind, int mode, int storage = 0);
+// Allow the blur kernels of the radii in the mask (bit R) their shared memory.
+cudaError_t blur_set_attributes(unsigned radii);
 
 // Detection (detect.cu)
 // pdl: launch as a programmatic dependent of the previous kernel on s.
