@@ -208,7 +208,7 @@ sift_status sift_match(sift_handle *h, const float *desc_a, int n_a, const float
     if (sift::match_set_attributes() != cudaSuccess) return fail(h, SIFT_E_CUDA, "matcher attributes");
     h->match_attr = true;
   }
-  const size_t need = sift::match_workspace_bytes(n_a, n_b);
+  const size_t need = sift::match_workspace_bytes(n_a, n_b, h->eng->sm_count());
   if (need > h->match_cap) {
     if (h->match_ws) cudaFreeAsync(h->match_ws, h->match_stream ? h->match_stream : s);
     h->match_ws = nullptr;
@@ -220,7 +220,8 @@ sift_status sift_match(sift_handle *h, const float *desc_a, int n_a, const float
     h->match_cap = need;
   }
   h->match_stream = s;
-  const cudaError_t e = sift::launch_match(desc_a, n_a, desc_b, n_b, ratio, h->match_ws, out_match_a, s);
+  const cudaError_t e = sift::launch_match(desc_a, n_a, desc_b, n_b, ratio, h->match_ws, out_match_a,
+                                            h->eng->sm_count(), s);
   if (e != cudaSuccess) return fail(h, SIFT_E_CUDA, std::string("matcher: ") + cudaGetErrorString(e));
   return SIFT_OK;
 }

@@ -266,10 +266,10 @@ cudaError_t launch_magsac(const float *xa, const float *xb, int n, const int *sa
                           float *score_out, unsigned char *inliers, float *scores_out);
 cudaError_t descriptor_set_attributes();
 // Matcher (match.cu)
-size_t match_workspace_bytes(int n_a, int n_b);
+size_t match_workspace_bytes(int n_a, int n_b, int n_sm);
 cudaError_t match_set_attributes();
 cudaError_t launch_match(const float *A, int n_a, const float *B, int n_b, float ratio, void *ws,
-                         int *out, cudaStream_t s);
+                         int *out, int n_sm, cudaStream_t s);
 int descriptor_smem_bytes();
 
 }  // namespace sift
