@@ -405,22 +405,8 @@ sift_status sift_build_pyramid(sift_handle *h, const float *img_dev, int H, int 
   h->n_parts = 0;
   st = h->eng->run_pyramid(in, s);
   if (st != SIFT_OK) return pass(h, st);
-  const sift::Desc &hd = h->eng->host_desc();
-  const int L = h->eng->params().n_scales + 3;
-  const float *pyr = reinterpret_cast<const float *>(h->eng->workspace() + h->eng->layout().pyr);
-  size_t off = 0;
-  for (int o = 0; o < no; o++) {
-    const sift::OctDev &od = hd.oct[o];
-    for (int l = 0; l < L; l++) {
-      const float *lv = od.half ? reinterpret_cast<const float *>(
-                                      reinterpret_cast<const __half *>(pyr + od.lvl) + (size_t)l * od.lstride)
-                                : pyr + od.lvl + (size_t)l * od.lstride;
-      cudaError_t e = sift::launch_export_level(lv, od.half != 0, od.pitch, od.H, od.W,
-                                                out_dev + off, s);
-      if (e != cudaSuccess) return fail(h, SIFT_E_CUDA, cudaGetErrorString(e));
-      off += (size_t)od.H * od.W;
-    }
-  }
+  const cudaError_t e = sift::launch_export(h->eng->device_desc(), out_dev, h->eng->sm_count(), s);
+  if (e != cudaSuccess) return fail(h, SIFT_E_CUDA, cudaGetErrorString(e));
   return SIFT_OK;
 }
 

@@ -469,49 +469,8 @@ int Engine::level_grid(int o, int l, int kind) const {
   return grid_blur(lvl_R_[l], kind, o > 0 && l == 1 ? 3 : 0, tun_.blur_ctas[o], storage(o, l));
 }
 
-cudaError_t Engine::enqueue_pyramid(cudaStream_t s, int M, int modes, std::vector<ProfRec> *prof) {
-  cudaError_t e = cudaSuccess;
-  auto rec = [&](int cls, auto &&fn) {
-    if (e != cudaSuccess) return;
-    ProfRec r{nullptr, nullptr, cls};
-    if (prof) {
-      cudaEventCreate(&r.a);
-      cudaEventCreate(&r.b);
-      e = cudaEventRecordWithFlags(r.a, s, cudaEventRecordExternal);
-    }
-    if (e == cudaSuccess) e = fn();
-    if (prof && e == cudaSuccess) {
-      e = cudaEventRecordWithFlags(r.b, s, cudaEventRecordExternal);
-      prof->push_back(r);
-    }
-  };
-  const Desc *d = ddesc_;
-  for (int o = 0; o < M; o++) {
-    if (o == 0) {
-      // One base launch per mode present (bit m of modes: images with up = m).
-      for (int m = 1; m >= 0; m--) {
-        if (!(modes >> m & 1)) continue;
-        rec(PC_BASE, [&] {
-          return launch_base_blur(d, base_R_[m], base_t_[m], m == 1,
-                                  grid_blur(base_R_[m], TK_BLUR32, m == 1 ? 2 : 1), s);
-        });
-      }
-    }
-    // Octaves above 0: the level-1 launch also produces level 0 by decimating
-    // level S of the previous octave (no separate decimation pass).
-    for (int l = 1; l <= S_ + 2; l++) {
-      const int kind = storage(o, l) ? TK_BLUR32 : tun_.lvl_kind[o][l];
-      rec(PC_BLUR, [&] {
-        return launch_level_blur(d, o, l, lvl_R_[l], lvl_t_[l], kind, level_grid(o, l, kind), s,
-                                 o > 0 && l == 1, true, storage(o, l));
-      });
-    }
-  }
-  return e;
-}
-
 cudaError_t Engine::enqueue_all(cudaStream_t s, int M, int modes, std::vector<ProfRec> *prof,
-                                bool fork) {
+                                bool fork, bool pyramid_only) {
   cudaError_t e = cudaSuccess;
   kernels_ = 0;
   auto rec_on = [&](cudaStream_t st, int cls, auto &&fn, int nk = 1) {
@@ -536,6 +495,12 @@ cudaError_t Engine::enqueue_all(cudaStream_t s, int M, int modes, std::vector<Pr
   // branches join the main stream before the last octave's scan, which the
   // keypoint stages follow.
   fork = fork && side_[0] != nullptr && M > 1;
+  auto join = [&] {
+    for (int k = 0; k < kSides && k < M - 1; k++) {
+      if (e == cudaSuccess) e = cudaEventRecord(join_ev_[k], side_[k]);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(s, join_ev_[k], 0);
+    }
+  };
   const Desc *d = ddesc_;
   const int g4 = n_sm_ * 4;
   const int ext_grid = grid_of(ext_max_, tun_.ext_ctas);
@@ -569,18 +534,18 @@ cudaError_t Engine::enqueue_all(cudaStream_t s, int M, int modes, std::vector<Pr
                                  storage(o, l));
       });
     }
-    if (branch) {
+    if (pyramid_only) {
+      if (fork && !branch) join();
+    } else if (branch) {
       rec_on(side, PC_EXTREMA, [&] { return launch_extrema(d, o, S_, ext_grid, side, true, half_octave(o)); });
     } else if (fork) {
-      for (int k = 0; k < kSides && k < M - 1; k++) {
-        if (e == cudaSuccess) e = cudaEventRecord(join_ev_[k], side_[k]);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, join_ev_[k], 0);
-      }
+      join();
       rec(PC_EXTREMA, [&] { return launch_extrema(d, o, S_, ext_grid, s, false, half_octave(o)); });
     } else {
       rec(PC_EXTREMA, [&] { return launch_extrema(d, o, S_, ext_grid, s, true, half_octave(o)); });
     }
   }
+  if (pyramid_only) return e;
   const int g2 = compact_grid();
   rec(PC_KEYPOINT, [&] { return launch_bm_compact(d, g2, s); });
   rec(PC_REFINE, [&] { return launch_refine(d, g4, s); });
@@ -608,22 +573,24 @@ void Engine::drop_graphs() {
   last_prof_ = nullptr;
 }
 
-sift_status Engine::get_graph(int M, int modes, cudaGraphExec_t *out) {
-  const int key = (M * 4 + modes) * 2 + (profiling_ ? 1 : 0);
+sift_status Engine::get_graph(int M, int modes, cudaGraphExec_t *out, bool pyramid_only) {
+  const bool prof = profiling_ && !pyramid_only;  // exports are not profiled
+  const int key = ((M * 4 + modes) * 2 + (prof ? 1 : 0)) * 2 + (pyramid_only ? 1 : 0);
   auto it = graphs_.find(key);
   if (it != graphs_.end()) {
     *out = it->second.exec;
+    if (pyramid_only) return SIFT_OK;
     last_prof_ = it->second.prof;
     last_kernels_ = it->second.kernels;
     return SIFT_OK;
   }
   GraphEntry ge;
-  if (profiling_) ge.prof = new std::vector<ProfRec>();
+  if (prof) ge.prof = new std::vector<ProfRec>();
   cudaError_t e = cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal);
   // The profiled graph (an event pair around every launch) keeps every launch
   // on one stream, so that each kernel's time is its own and not shared with a
   // concurrent branch.
-  cudaError_t e1 = e == cudaSuccess ? enqueue_all(cap_, M, modes, ge.prof, !profiling_) : e;
+  cudaError_t e1 = e == cudaSuccess ? enqueue_all(cap_, M, modes, ge.prof, !prof, pyramid_only) : e;
   cudaGraph_t g = nullptr;
   cudaError_t e2 = e == cudaSuccess ? cudaStreamEndCapture(cap_, &g) : e;
   cudaError_t e3 = (e1 == cudaSuccess && e2 == cudaSuccess) ? cudaGraphInstantiate(&ge.exec, g, 0)
@@ -638,6 +605,7 @@ sift_status Engine::get_graph(int M, int modes, cudaGraphExec_t *out) {
   ge.kernels = kernels_;
   graphs_[key] = ge;
   *out = ge.exec;
+  if (pyramid_only) return SIFT_OK;
   last_prof_ = ge.prof;
   last_kernels_ = ge.kernels;
   return SIFT_OK;
@@ -741,11 +709,13 @@ sift_status Engine::run_pyramid(const ImgIn &img, cudaStream_t s) {
   hd->pyr = reinterpret_cast<float *>(ws_ + lay.pyr);
   hd->bm = reinterpret_cast<uint32_t *>(ws_ + lay.bm);
   const size_t bytes = offsetof(Desc, oct) + (size_t)hd->img[0].n_oct * sizeof(OctDev);
-  cudaError_t e = cudaSuccess;
-  st = upload(hd, bytes, s);
-  if (e == cudaSuccess && st == SIFT_OK) e = enqueue_pyramid(s, M, base_modes(*hd), nullptr);
+  cudaGraphExec_t exec = nullptr;
+  st = get_graph(M, base_modes(*hd), &exec, true);
+  if (st == SIFT_OK) st = upload(hd, bytes, s);
+  if (st != SIFT_OK) return st;
+  cudaError_t e = cudaGraphLaunch(exec, s);
   if (e == cudaSuccess) e = cudaEventRecord(done_, s);
-  if (e != cudaSuccess || st != SIFT_OK) {
+  if (e != cudaSuccess) {
     err = std::string("pyramid launch failed: ") + cudaGetErrorString(e);
     return SIFT_E_CUDA;
   }
@@ -853,9 +823,9 @@ sift_status Engine::autotune(int H, int W, cudaStream_t s) {
   // from 32-row tiles everywhere in octave 0; a level switches to 64 rows only
   // if the stage gets at least 1% faster.
   auto time_stage = [&]() -> float {
-    for (int w = 0; w < 2; w++) enqueue_pyramid(s, M, modes, nullptr);
+    for (int w = 0; w < 2; w++) enqueue_all(s, M, modes, nullptr, false, true);
     cudaEventRecord(a, s);
-    for (int r = 0; r < 5; r++) enqueue_pyramid(s, M, modes, nullptr);
+    for (int r = 0; r < 5; r++) enqueue_all(s, M, modes, nullptr, false, true);
     cudaEventRecord(b, s);
     cudaEventSynchronize(b);
     float ms = 0.f;

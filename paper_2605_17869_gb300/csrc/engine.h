@@ -153,12 +153,11 @@ class Engine {
   sift_status ensure_workspace(size_t bytes, cudaStream_t s);
   sift_status upload(Desc *hd, size_t bytes, cudaStream_t s);
   // modes: bit 0 set if an image is processed as is, bit 1 if one is magnified.
-  cudaError_t enqueue_pyramid(cudaStream_t s, int max_oct, int modes, std::vector<struct ProfRec> *prof);
   // fork: run the extrema scans of all but the last octave on a side branch
   // (graph capture only; the allocation-free path runs everything in order).
   cudaError_t enqueue_all(cudaStream_t s, int max_oct, int modes, std::vector<struct ProfRec> *prof,
-                          bool fork = false);
-  sift_status get_graph(int max_oct, int modes, cudaGraphExec_t *out);
+                          bool fork = false, bool pyramid_only = false);
+  sift_status get_graph(int max_oct, int modes, cudaGraphExec_t *out, bool pyramid_only = false);
   void drop_graphs();
   int grid_blur(int R, int kind, int mode, int ctas = 0, int storage = 0) const;
   // Grid of the launch that writes level l of octave o in row class `kind`.

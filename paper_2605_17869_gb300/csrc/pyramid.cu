@@ -333,22 +333,47 @@ cudaError_t launch_level_blur(const Desc *d, int oct, int lvl_out, int R, const 
 }
 
 namespace {
-// One pyramid level copied out as a dense H x W FP32 plane (binary16 levels
-// widened), for the pyramid export.
-__global__ void k_export_level(const float *__restrict__ src, int half, int pitch, int H, int W,
-                               float *__restrict__ dst) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-  if (x >= W || y >= H) return;
-  const long long i = (long long)y * pitch + x;
-  dst[(long long)y * W + x] =
-      half ? __half2float(reinterpret_cast<const __half *>(src)[i]) : src[i];
+// The whole pyramid of image 0 copied out as dense H x W FP32 planes (binary16
+// levels widened), octave by octave, level by level: a warp copies rows, 16 bytes
+// per lane where the output row allows it, four loads in flight. One launch: it was
+// one per level, 42 of them for 1920 x 1080, and the host's launches were the
+// call's bound.
+__global__ void __launch_bounds__(256) k_export(const Desc *__restrict__ d, float *__restrict__ out) {
+  const int n_oct = d->img[0].n_oct, L = d->n_scales + 3;
+  const int lane = threadIdx.x & 31;
+  int o = 0, first = 0;  // octave of row r and its first row
+  long long off = 0;     // the octave's offset in `out`
+  OctDev od = d->oct[d->img[0].oct0];
+  for (int r = blockIdx.x * 8 + (threadIdx.x >> 5);; r += gridDim.x * 8) {
+    while (r - first >= L * od.H) {
+      first += L * od.H;
+      off += (long long)L * od.H * od.W;
+      if (++o >= n_oct) return;
+      od = d->oct[d->img[0].oct0 + o];
+    }
+    const int rr = r - first, l = rr / od.H, y = rr - l * od.H;
+    const long long se = (long long)l * od.lstride + (long long)y * od.pitch;
+    float *dst = out + off + (long long)rr * od.W;
+    const float *lv = d->pyr + od.lvl;
+    if (od.half) {
+      const __half *src = reinterpret_cast<const __half *>(lv) + se;
+#pragma unroll 4
+      for (int c = lane; c < od.W; c += 32) dst[c] = __half2float(src[c]);
+    } else if ((od.W & 3) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
+      const float4 *src = reinterpret_cast<const float4 *>(lv + se);
+#pragma unroll 4
+      for (int c = lane; c < od.W / 4; c += 32) reinterpret_cast<float4 *>(dst)[c] = src[c];
+    } else {
+      const float *src = lv + se;
+#pragma unroll 4
+      for (int c = lane; c < od.W; c += 32) dst[c] = src[c];
+    }
+  }
 }
 }  // namespace
 
-cudaError_t launch_export_level(const float *src, bool half, int pitch, int H, int W, float *dst,
-                                cudaStream_t s) {
-  return launch_plain(k_export_level, dim3((W + 127) / 128, H), 128, 0, s, src, half ? 1 : 0,
-                      pitch, H, W, dst);
+cudaError_t launch_export(const Desc *d, float *out, int n_sm, cudaStream_t s) {
+  return launch_plain(k_export, n_sm * 8, 256, 0, s, d, out);
 }
 
 cudaError_t launch_base_blur(const Desc *d, int R, const BlurTaps &t, bool upsample, int grid,

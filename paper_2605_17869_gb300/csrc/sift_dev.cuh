@@ -217,10 +217,8 @@ cudaError_t launch_base_blur(const Desc *d, int R, const BlurTaps &t, bool upsam
 cudaError_t launch_level_blur(const Desc *d, int oct, int lvl_out, int R, const BlurTaps &t,
                               int th_kind, int grid, cudaStream_t s,
                               bool from_prev_octave = false, bool pdl = true, int storage = 0);
-// Copy one pyramid level (src: the level's first element, `half` for binary16)
-// into a dense H x W FP32 plane.
-cudaError_t launch_export_level(const float *src, bool half, int pitch, int H, int W, float *dst,
-                                cudaStream_t s);
+// Copy the pyramid of image 0 into dense FP32 planes.
+cudaError_t launch_export(const Desc *d, float *out, int n_sm, cudaStream_t s);
 // Rows of a tile of a row class.
 int blur_tile_rows(int th_kind);
 // mode: 0 level, 1 base as is, 2 magnified base, 3 level 1 from the previous octave.
