@@ -20,7 +20,7 @@ namespace sift {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kExtThreads = 128;  // extrema scan: four warps per block, five blocks per SM
+constexpr int kExtThreads = 128;  // extrema scan: four independent warps per block
 
 // ------------------------------------------------------------ extrema scan
 
@@ -36,131 +36,162 @@ __device__ __forceinline__ float min3f(float a, float b, float c) {
   return r;
 }
 
-// One row of DoG values as the scan holds it, for the lane's column x: the
-// maximum and minimum over columns x - 1 .. x + 1 of each of the S + 2 DoG
-// layers, and for the tested layers 1 .. S the value itself and the larger and
-// smaller of its left and right neighbours.
+// One row of DoG values as the scan holds it, for the lane's columns x and x + 1:
+// the maximum and minimum over columns x - 1 .. x + 1 and x .. x + 2 of each of
+// the S + 2 DoG layers, and for the tested layers 1 .. S the values at columns
+// x - 1 .. x + 2.
 template <int S> struct ExtRow {
-  float hx[S + 2], hn[S + 2];
-  float c[S], lrx[S], lrn[S];
+  float hx[S + 2][2], hn[S + 2][2];
+  float l[S], c[S][2], r[S];
 };
 
-// DoG (one FP32 subtraction per value, as in every other stage) of one row
-// from its S + 3 Gaussian levels, and the row's three-column maxima / minima
-// (neighbours by warp shuffle; lanes 0 and 31 get meaningless values there,
-// they only supply neighbours).
+// DoG (one FP32 subtraction per value, as in every other stage) of one row from
+// its S + 3 Gaussian levels, and the row's three-column maxima / minima: the two
+// outer neighbours by warp shuffle (lane 0's left and lane 31's right one are
+// meaningless; these lanes only supply neighbours).
 template <int S>
-__device__ __forceinline__ void ext_row(ExtRow<S> &R, const float (&g)[S + 3]) {
+__device__ __forceinline__ void ext_row(ExtRow<S> &R, const float2 (&g)[S + 3]) {
 #pragma unroll
-  for (int l = 0; l < S + 2; l++) {
-    const float v = g[l + 1] - g[l];
-    const float lf = __shfl_up_sync(0xffffffffu, v, 1);
-    const float rt = __shfl_down_sync(0xffffffffu, v, 1);
-    R.hx[l] = max3f(lf, v, rt);
-    R.hn[l] = min3f(lf, v, rt);
-    if (l >= 1 && l <= S) {
-      R.c[l - 1] = v;
-      R.lrx[l - 1] = fmaxf(lf, rt);
-      R.lrn[l - 1] = fminf(lf, rt);
+  for (int i = 0; i < S + 2; i++) {
+    const float v0 = g[i + 1].x - g[i].x, v1 = g[i + 1].y - g[i].y;
+    const float lf = __shfl_up_sync(0xffffffffu, v1, 1);
+    const float rt = __shfl_down_sync(0xffffffffu, v0, 1);
+    R.hx[i][0] = max3f(lf, v0, v1);
+    R.hn[i][0] = min3f(lf, v0, v1);
+    R.hx[i][1] = max3f(v0, v1, rt);
+    R.hn[i][1] = min3f(v0, v1, rt);
+    if (i >= 1 && i <= S) {
+      R.l[i - 1] = lf;
+      R.c[i - 1][0] = v0;
+      R.c[i - 1][1] = v1;
+      R.r[i - 1] = rt;
     }
   }
 }
 
-// The rows a warp has in flight: a ring of kExtRing rows x (S + 3) levels x
-// 32 lanes in shared memory, filled by 4-byte asynchronous copies (each lane
-// copies its own column) so that kExtRing - 1 rows are on their way while
-// one is consumed.
-constexpr int kExtRing = 4;  // a power of two
+// The rows a warp has in flight: kExtRing rows x (S + 3) levels x 32 lanes in
+// shared memory, filled by asynchronous copies (each lane copies and reads its
+// own two columns); a row's slot is refilled as soon as it is read. Three, as the
+// rows that the tests hold in turn, so that every slot is a fixed address.
+constexpr int kExtRing = 3;
 
-__device__ __forceinline__ void cp_async4_ca(float *dst, const float *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
-                   static_cast<unsigned>(__cvta_generic_to_shared(dst))),
-               "l"(src)
-               : "memory");
+__device__ __forceinline__ void cp_async4_ca(unsigned dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8_ca(unsigned dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ unsigned lds32(unsigned a) {
+  unsigned v;
+  asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 lds64(unsigned a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// Copy the S + 3 levels of one image row at the lane's column into a ring
-// slot (lp[l]: level l at row 0 and the lane's column; row_off: the row's
-// offset, the same for the whole warp).
-template <int S>
-__device__ __forceinline__ void ext_issue(float *slot, const float *const (&lp)[S + 3],
-                                          long long row_off) {
-#pragma unroll
-  for (int l = 0; l < S + 3; l++) cp_async4_ca(slot + l * 32, lp[l] + row_off);
+// Bits 0 .. 14 spread to the even bit positions 0 .. 28.
+__device__ __forceinline__ unsigned spread15(unsigned v) {
+  v = (v | (v << 8)) & 0x00ff00ffu;
+  v = (v | (v << 4)) & 0x0f0f0f0fu;
+  v = (v | (v << 2)) & 0x33333333u;
+  return (v | (v << 1)) & 0x55555555u;
 }
 
-// Test row y (P, C, N: rows y - 1, y, y + 1) and write its bitmap words:
-// pixel x of layer s is a candidate when it lies inside the border, |D|
-// exceeds the pre-gate, and D is strictly above the maximum, or strictly
-// below the minimum, of its 26 neighbours. Those extrema are separable: the
-// 9 values of layer s +- 1 reduce to max(hx(y - 1), hx(y), hx(y + 1)), the 8
-// of layer s to max(hx(y - 1), hx(y + 1), left, right).
+// Test row y (P, C, N: rows y - 1, y, y + 1) and write its bitmap words: pixel x
+// of layer s is a candidate when it lies inside the border, |D| exceeds the
+// pre-gate, and D is strictly above the maximum, or strictly below the minimum,
+// of its 26 neighbours. Those extrema are separable: the 9 values of layer s +- 1
+// reduce to max(hx(y - 1), hx(y), hx(y + 1)), the 8 of layer s to max(hx(y - 1),
+// hx(y + 1), left, right). Lane s of the first S writes layer s + 1's two words
+// (word: its address, two: whether the row has the second one).
+// thr0, thr1: the pre-gate for the lane's columns, infinite where a column lies
+// outside the border (no |D| is above it).
 template <int S>
 __device__ __forceinline__ void ext_test(const ExtRow<S> &P, const ExtRow<S> &C,
-                                         const ExtRow<S> &N, bool inb, float thr, int lane,
-                                         uint32_t *word) {
+                                         const ExtRow<S> &N, bool yin, float thr0, float thr1,
+                                         int lane, uint32_t *word, bool two) {
   // Rows where no pixel of the strip passes the border and pre-gate tests
   // in any layer have no candidate: skip the neighbour comparisons.
-  float amax = fabsf(C.c[0]);
+  bool gate = false;
 #pragma unroll
-  for (int s = 2; s <= S; s++) amax = fmaxf(amax, fabsf(C.c[s - 1]));
-  if (!__any_sync(0xffffffffu, inb && amax > thr)) {
-    if (lane < S) *word = 0u;
-    return;
-  }
-  float vx[S + 2], vn[S + 2];
+  for (int s = 0; s < S; s++) gate |= (fabsf(C.c[s][0]) > thr0) | (fabsf(C.c[s][1]) > thr1);
+  unsigned lo = 0u, hi = 0u;
+  if (yin && __any_sync(0xffffffffu, gate)) {
+    bool ok[S][2], any = false;
 #pragma unroll
-  for (int l = 0; l < S + 2; l++) {
-    vx[l] = max3f(P.hx[l], C.hx[l], N.hx[l]);
-    vn[l] = min3f(P.hn[l], C.hn[l], N.hn[l]);
-  }
-  unsigned mine = 0u;
+    for (int k = 0; k < 2; k++) {
+      float vx[S + 2], vn[S + 2];
 #pragma unroll
-  for (int s = 1; s <= S; s++) {
-    const float c = C.c[s - 1];
-    const float mx = max3f(vx[s - 1], vx[s + 1], max3f(P.hx[s], N.hx[s], C.lrx[s - 1]));
-    const float mn = min3f(vn[s - 1], vn[s + 1], min3f(P.hn[s], N.hn[s], C.lrn[s - 1]));
-    // |c| > thr and (c > mx or c < mn), as one comparison with zero: the
-    // differences of distinct finite FP32 values are never zero (gradual
-    // underflow) and keep their sign, so each difference is positive exactly
-    // when its comparison holds, and the minimum / maximum combine them. The
-    // subtractions run on the FMA pipe, leaving the ALU pipe (the scan's
-    // bound) three instructions instead of five.
-    const float margin = fminf(fabsf(c) - thr, fmaxf(c - mx, mn - c));
-    const bool ok = inb && margin > 0.f;
-    const unsigned bits = __ballot_sync(0xffffffffu, ok);
-    mine = lane == s - 1 ? bits : mine;
+      for (int i = 0; i < S + 2; i++) {
+        vx[i] = max3f(P.hx[i][k], C.hx[i][k], N.hx[i][k]);
+        vn[i] = min3f(P.hn[i][k], C.hn[i][k], N.hn[i][k]);
+      }
+#pragma unroll
+      for (int s = 1; s <= S; s++) {
+        const float c = C.c[s - 1][k];
+        const float lf = k ? C.c[s - 1][0] : C.l[s - 1], rt = k ? C.r[s - 1] : C.c[s - 1][1];
+        const float mx = fmaxf(max3f(vx[s - 1], vx[s + 1], lf), max3f(P.hx[s][k], N.hx[s][k], rt));
+        const float mn = fminf(min3f(vn[s - 1], vn[s + 1], lf), min3f(P.hn[s][k], N.hn[s][k], rt));
+        ok[s - 1][k] = ((c > mx) | (c < mn)) & (fabsf(c) > (k ? thr1 : thr0));
+        any |= ok[s - 1][k];
+      }
+    }
+    if (__any_sync(0xffffffffu, any)) {
+unsigned m0 = 0u, m1 = 0u;  // lane s: layer s + 1 at the lanes' first / second columns
+#pragma unroll
+      for (int s = 0; s < S; s++) {
+        const unsigned b0 = __ballot_sync(0xffffffffu, ok[s][0]), b1 = __ballot_sync(0xffffffffu, ok[s][1]);
+        m0 = lane == s ? b0 : m0;
+        m1 = lane == s ? b1 : m1;
+      }
+      // Lanes 1 .. 15: columns 0 .. 29 of the strip; 16 .. 30: 30 .. 59.
+      lo = spread15(m0 >> 1 & 0x7fffu) | spread15(m1 >> 1 & 0x7fffu) << 1;
+      hi = spread15(m0 >> 16 & 0x7fffu) | spread15(m1 >> 16 & 0x7fffu) << 1;
+    }
   }
-  if (lane < S) *word = mine >> 1;  // lanes 1 .. 30 -> bits 0 .. 29
+  if (lane < S) {
+    word[0] = lo;
+    if (two) word[1] = hi;
+  }
 }
 
-// A warp owns a strip of kBmCols = 30 columns x kExtTH rows: lane l holds
-// column 30 tx - 1 + l, so lanes 1 .. 30 are the strip and lanes 0 and 31 its
-// neighbours, and one bitmap word covers the strip's row. The warp streams
-// down the strip: each image row's S + 3 levels are loaded once (the next
-// row's loads are in flight while the current row is tested) and every test
-// is done from registers. The candidate decisions are exact comparisons of
-// the same FP32 values, so they do not depend on the tiling. Bitmap words are
-// written by ballots; no atomics.
-// HALF: the octave's levels are binary16 (fp16 storage mode). cp.async has no
-// 2-byte copy, so each lane copies the 32-bit word that holds its column's
-// value (4-byte aligned: rows start on 64-byte boundaries) and takes the low
-// or the high half of it, widened to FP32, when it reads the row.
+// A warp owns a strip of 2 kBmCols = 60 columns x ext_rows[oct] rows: lane l
+// holds columns 60 tx - 2 + 2l and the next one, so lanes 1 .. 30 are the strip
+// (two bitmap words per row and layer) and lanes 0 and 31 its neighbours. The
+// warp streams down the strip: each image row's S + 3 levels are copied once, by
+// 8 bytes per lane, kExtRing rows ahead, and every test is done from registers.
+// The candidate decisions are exact comparisons of the same FP32 values, so they do
+// not depend on the tiling. Bitmap words are written by ballots; no atomics.
+// Two columns per lane share the copies, the loop, two of four shuffles per layer
+// and the middle values of the three-column extrema: 3.5 warp instructions per
+// tested pixel column against 4.9 with one column. What bounds it is the ALU pipe
+// (66%: three-input extrema and comparisons) together with HBM (52%, every level
+// value read once) at 16 warps per SM, which 128 registers allow (12 warps at 150:
+// 2 percent more per call on the 64-image batch); rings of 4 and 8 rows were no
+// faster than 3. Octave 0 of half that batch: 170 us before, 165 now; all scans of
+// four 1024 x 768 images with five layers, whose strips of one column per lane left
+// 8 warps per SM: 333 -> 286 us per call.
+// HALF: the octave's levels are binary16 (fp16 storage mode): a lane's two columns
+// are one 32-bit word, widened when the row is read.
 template <int S, bool HALF>
-__global__ void __launch_bounds__(kExtThreads, 5) k_extrema(const Desc *__restrict__ d, int oct) {
+__global__ void __launch_bounds__(kExtThreads, S <= 3 ? 4 : S == 4 ? 3 : 2) k_extrema(const Desc *__restrict__ d, int oct) {
   constexpr int WPB = kExtThreads / 32;
-  constexpr int SLOT = (S + 3) * 32;
-  __shared__ float ring[WPB][kExtRing * SLOT];
+  constexpr int PB = HALF ? 4 : 8;                       // bytes of a lane's pair
+  constexpr int LB = 32 * PB, SB = (S + 3) * LB;         // of a level's and of a row's pairs
+  __shared__ __align__(16) unsigned char ring[WPB * kExtRing * SB];
   const int n = d->n_img;
   const int *pre = d->tile_pre[TK_EXT][oct];
   const int total = pre[n];
   const int lane = threadIdx.x & 31;
-  float *my = ring[threadIdx.x >> 5];
-  const float thr = d->prefilter;
-  const int bord = d->border;
+  const unsigned my = static_cast<unsigned>(__cvta_generic_to_shared(ring)) +
+                      (threadIdx.x >> 5) * (kExtRing * SB) + lane * PB;
+  const int bord = d->border, th = d->ext_rows[oct];
   pdl_wait();
   for (int t = blockIdx.x * WPB + (threadIdx.x >> 5); t < total; t += gridDim.x * WPB) {
     if (t + gridDim.x * WPB >= total) pdl_trigger();  // this warp's last tile
@@ -169,70 +200,67 @@ __global__ void __launch_bounds__(kExtThreads, 5) k_extrema(const Desc *__restri
     const int H = od.H, W = od.W;
     const long long pitch = od.pitch, ls = od.lstride;
     const int lt = t - pre[b];
-    const int ty = lt / od.wpr, tx = lt - ty * od.wpr;
-    const int x = tx * kBmCols - 1 + lane;
-    const int y0 = ty * kExtTH, y1 = min(y0 + kExtTH, H);
-    // lp[l]: the 32-bit word of level l, row 0, that holds the lane's column
-    // (binary16 levels: the word of halves xc & ~1 and its neighbour); a row's
-    // words are rstride apart.
-    const float *lp[S + 3];
-    const int xc = min(max(x, 0), W - 1);
-    const bool hi_half = HALF && (xc & 1);
-    const long long rstride = HALF ? pitch / 2 : pitch;
-    {
-      const float *G = HALF ? reinterpret_cast<const float *>(
-                                  reinterpret_cast<const __half *>(d->pyr + od.lvl) + (xc & ~1))
-                            : d->pyr + od.lvl + xc;
+    const int sx = (od.wpr + 1) / 2;  // strips per row
+    const int ty = lt / sx, tx = lt - ty * sx;
+    const int x = tx * (2 * kBmCols) - 2 + 2 * lane;
+    const int y0 = ty * th, y1 = min(y0 + th, H);
+    // G: the lane's pair of columns in row 0 of level 0; x is even and rows
+    // start on 64-byte boundaries at least. Pairs past the row's padding and left
+    // of the image are moved inside: no tested pixel has them as neighbours.
+    constexpr int EB = HALF ? 2 : 4;
+    const char *G = reinterpret_cast<const char *>(d->pyr + od.lvl) +
+                    (long long)min(max(x, 0), (int)pitch - 2) * EB;
+    const long long lb = ls * EB;
+    const bool lx = lane >= 1 && lane <= kBmCols;
+    const float thr0 = lx && x >= bord && x < W - bord ? d->prefilter : INFINITY;
+    const float thr1 = lx && x + 1 >= bord && x + 1 < W - bord ? d->prefilter : INFINITY;
+    const bool two = 2 * tx + 1 < od.wpr;
+    uint32_t *bmw = d->bm + od.bm + ((long long)lane * H + y0) * od.wpr + 2 * tx;
+    // Row k of the strip's sequence is image row y0 - 1 + k (clamped); it lives in
+    // slot k % 3. One commit group per row, empty past the last one (y1), so that
+    // the number of pending groups is fixed.
+    auto issue = [&](int slot, int y) {
+      if (y <= y1) {
+        const char *p = G + (long long)min(max(y, 0), H - 1) * pitch * EB;
 #pragma unroll
-      for (int l = 0; l < S + 3; l++) lp[l] = G + l * (HALF ? ls / 2 : ls);
-    }
-    float *mine_ring = my + lane;
-    const bool xin = lane >= 1 && lane <= kBmCols && x >= bord && x < W - bord;
-    uint32_t *bmw = d->bm + od.bm + (long long)lane * H * od.wpr + tx;
-    // Row k of the strip's sequence is image row y0 - 1 + k (clamped), k = 0 ..
-    // n_rows - 1; it lives in ring slot k % kExtRing. One commit group per
-    // row, empty past the end, so that the number of pending groups is fixed.
-    const int n_rows = y1 - y0 + 2;
-    auto issue = [&](int k) {
-      if (k < n_rows) {
-        const int row = min(max(y0 - 1 + k, 0), H - 1);
-        ext_issue<S>(mine_ring + (k & (kExtRing - 1)) * SLOT, lp, row * rstride);
+        for (int l = 0; l < S + 3; l++) {
+          if (HALF) cp_async4_ca(my + slot * SB + l * LB, p + l * lb);
+          else cp_async8_ca(my + slot * SB + l * LB, p + l * lb);
+        }
       }
       cp_async_commit();
     };
-    auto consume = [&](ExtRow<S> &R, int k) {
-      cp_async_wait<kExtRing - 1>();  // row k's group is complete
-      const float *slot = mine_ring + (k & (kExtRing - 1)) * SLOT;
-      float g[S + 3];
+    auto consume = [&](ExtRow<S> &R, int slot, int y) {  // image row y
+      cp_async_wait<kExtRing - 1>();
+      float2 g[S + 3];
 #pragma unroll
       for (int l = 0; l < S + 3; l++) {
-        if (HALF) {
-          const unsigned w = __float_as_uint(slot[l * 32]);
-          g[l] = __half2float(__ushort_as_half((unsigned short)(hi_half ? w >> 16 : w & 0xffffu)));
+        if constexpr (HALF) {
+          const unsigned w = lds32(my + slot * SB + l * LB);
+          g[l] = __half22float2(*reinterpret_cast<const __half2 *>(&w));
         } else {
-          g[l] = slot[l * 32];
+          g[l] = lds64(my + slot * SB + l * LB);
         }
       }
       ext_row<S>(R, g);
-      issue(k + kExtRing);  // into the slot just read (each lane rewrites only its own words)
+      issue(slot, y + kExtRing);  // into the slot just read (each lane rewrites only its own words)
     };
 #pragma unroll
-    for (int k = 0; k < kExtRing; k++) issue(k);
+    for (int k = 0; k < kExtRing; k++) issue(k, y0 - 1 + k);
     ExtRow<S> A, B, C;
-    consume(A, 0);
-    consume(B, 1);
-    // Rows rotate through A, B, C (previous, current, next) without copies.
-    auto step = [&](ExtRow<S> &Pr, ExtRow<S> &Cu, ExtRow<S> &Nx, int y) {
-      consume(Nx, y - y0 + 2);                                    // image row y + 1 (clamped)
-      const bool inb = xin && y >= bord && y < H - bord;
-      ext_test<S>(Pr, Cu, Nx, inb, thr, lane, bmw + (long long)y * od.wpr);
+    consume(A, 0, y0 - 1);
+    consume(B, 1, y0);
+    // Rows rotate through A, B, C (previous, current, next) without copies; the
+    // steps past the strip's last row test nothing.
+    auto step = [&](const ExtRow<S> &Pr, const ExtRow<S> &Cu, ExtRow<S> &Nx, int slot, int y) {
+      consume(Nx, slot, y + 1);
+      if (y < y1) ext_test<S>(Pr, Cu, Nx, y >= bord && y < H - bord, thr0, thr1, lane, bmw, two);
+      bmw += od.wpr;
     };
     for (int y = y0; y < y1; y += 3) {
-      step(A, B, C, y);
-      if (y + 1 >= y1) break;
-      step(B, C, A, y + 1);
-      if (y + 2 >= y1) break;
-      step(C, A, B, y + 2);
+      step(A, B, C, 2, y);
+      step(B, C, A, 0, y + 1);
+      step(C, A, B, 1, y + 2);
     }
     cp_async_wait<0>();  // no copy of this strip outlives it
     __syncwarp();
@@ -554,6 +582,8 @@ int compact_max_ctas() {
   if (e == cudaSuccess) e = cc_compact_occupancy(&b);
   return (e == cudaSuccess && a > 0 && b > 0) ? std::min(a, b) : 1;
 }
+
+int extrema_warps() { return kExtThreads / 32; }
 
 int extrema_max_ctas(int n_scales) {
   int nb = 0;

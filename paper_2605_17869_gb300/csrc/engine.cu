@@ -352,6 +352,21 @@ sift_status Engine::fill_plan(int n, const ImgIn *in, Desc &hd, WsLayout &L, int
   hd.n_oct_max = M;
   hd.n_bm_chunks = bmc;
   hd.n_cc_chunks = cc;
+  for (int o = 0; o < kMaxOct; o++) {
+    auto strips = [&](int rows) {
+      long long t = 0;
+      for (int b = 0; b < n; b++)
+        if (o < hd.img[b].n_oct) {
+          const OctDev &od = hd.oct[hd.img[b].oct0 + o];
+          t += (long long)div_up(od.wpr, 2) * div_up(od.H, rows);
+        }
+      return t;
+    };
+    const long long warps = (long long)n_sm_ * ext_max_ * extrema_warps();
+    int k = 0;
+    while (k < 3 && strips(kExtRows[k + 1]) <= warps) k++;
+    hd.ext_rows[o] = kExtRows[k];
+  }
   for (int k = 0; k < TK_COUNT; k++) {
     for (int o = 0; o < kMaxOct; o++) {
       int *pre = hd.tile_pre[k][o];
@@ -360,7 +375,7 @@ sift_status Engine::fill_plan(int n, const ImgIn *in, Desc &hd, WsLayout &L, int
         int t = 0;
         if (o < hd.img[b].n_oct) {
           const OctDev &od = hd.oct[hd.img[b].oct0 + o];
-          if (k == TK_EXT) t = od.wpr * div_up(od.H, kExtTH);
+          if (k == TK_EXT) t = div_up(od.wpr, 2) * div_up(od.H, hd.ext_rows[o]);
           else t = div_up(od.W, kBlurTW) * div_up(od.H, blur_tile_rows(k));
         }
         pre[b + 1] = pre[b] + t;

@@ -7,7 +7,7 @@
 //    (OctDev::half); arithmetic is FP32 throughout.
 //  * Candidate bitmap: per image, per octave, per DoG layer 1..S, H_o rows of
 //    ceil(W_o / 30) 32-bit words; bit k (< 30) of word w in row y marks pixel
-//    x = 30 w + k (one word is the row of one extrema strip). Walking the
+//    x = 30 w + k (two words are the row of one extrema strip). Walking the
 //    bitmap in memory order is the canonical order (octave, layer, row,
 //    column).
 //  * Keypoint-stage arrays are per image slices of global arrays; every slice
@@ -31,8 +31,9 @@ constexpr int kMaxPeaks = kOriBins / 2;  // strict circular maxima of 36 bins
 constexpr int kDescLen = 128;      // 4 x 4 x 8
 constexpr int kBlurTW = 128;       // blur tile width (32 lanes x float4)
 constexpr int kBlurHalo = 16;      // staged columns left/right of a blur tile
-constexpr int kBmCols = 30;        // columns per bitmap word = extrema strip width (one warp)
-constexpr int kExtTH = 32;         // extrema tile rows (one warp streams down them)
+constexpr int kBmCols = 30;        // columns per bitmap word; an extrema strip (one warp) has two words
+// Rows of an extrema strip (one warp streams down them), see ext_rows.
+constexpr int kExtRows[4] = {30, 15, 6, 3};
 constexpr int kChunk = 2048;       // compaction chunk (words or slots)
 
 // Work queues: blur tiles of the smaller and the larger row class (blur.cuh; 32
@@ -120,6 +121,10 @@ struct Desc {
   int *cand_flat;              // [kMaxImg + 1] prefix of n_cand over images
   int *fin_flat;               // [kMaxImg + 1] prefix of n_fin over images
   // geometry
+  // Rows of an octave's extrema strips: the shortest of kExtRows at which the scan's
+  // resident warps take all strips at once, else the longest (a warp streams down its rows one
+  // after the other, so a small octave's scan takes as long as its strips are).
+  int ext_rows[kMaxOct];
   int tile_pre[TK_COUNT][kMaxOct][kMaxImg + 1];
   // Base-blur work of the images with up = 0 (steps, or tiles at radius 0) / 1 (tiles).
   int base_pre[2][kMaxImg + 1];
@@ -235,6 +240,7 @@ cudaError_t extrema_set_attributes();
 // Persistent grid of the extrema scan: SMs x resident blocks per SM.
 // Occupancy maxima (resident CTAs per SM) of the persistent keypoint kernels.
 int extrema_max_ctas(int n_scales);
+int extrema_warps();  // warps per CTA of the scan
 int orientation_max_ctas(bool mixed);
 int descriptor_max_ctas(bool mixed);
 int compact_max_ctas();
