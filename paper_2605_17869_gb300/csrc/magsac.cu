@@ -1,9 +1,11 @@
 // GPU MAGSAC++ homography verification (§3.6 "GPU MAGSAC++").
 //
-// Hypotheses: one thread per minimal sample of 4 correspondences fits the
-// homography by the normalised DLT in FP64. Each image's 4 points are moved to
-// centroid 0 and mean distance sqrt(2). The 8 x 8 system of the DLT with
-// h33 = 1 is then solved by Gaussian elimination with partial pivoting, and the
+// Hypotheses: eight lanes per minimal sample of 4 correspondences fit the
+// homography by the normalised DLT in FP64, one lane per point, then per triangle,
+// per equation and per entry. Each image's 4 points are moved to centroid 0 and
+// mean distance sqrt(2). The 8 x 8 system of the DLT with h33 = 1 is then solved by
+// Gaussian elimination with partial pivoting (rows stay in their lanes, their
+// positions are exchanged), and the
 // result is de-normalised and scaled to H[2][2] = 1. A sample is degenerate
 // (score +inf) in four cases:
 //   - an index lies outside [0, n);
@@ -26,8 +28,9 @@
 // order, and the block combines the threads in a fixed tree: the scores are
 // bitwise reproducible.
 //
-// Selection: one block takes the smallest score (ties to the smaller index)
-// and marks the inliers of its model (r <= k sigma_max).
+// Selection: every block takes the smallest score (ties to the smaller index),
+// the first one writes it out, and each marks its share of the inliers of its
+// model (r <= k sigma_max).
 #include <algorithm>
 #include <cmath>
 
@@ -37,7 +40,7 @@ namespace sift {
 
 namespace {
 
-constexpr int kFitThreads = 32;  // most FP64 solver threads per block
+constexpr int kFitThreads = 32;  // four hypotheses per block: blocks spread over the SMs
 constexpr int kScoreThreads = 256;
 constexpr int kSelectThreads = 1024;
 
@@ -70,178 +73,159 @@ __device__ __forceinline__ float transfer_r2(const float *H, float2 a, float2 b)
   return dx * dx + dy * dy;
 }
 
-// Hartley normalisation of 4 points in place; returns (s, cx, cy).
-__device__ void normalise4(double p[4][2], double *s, double *cx, double *cy) {
-  double mx = 0.0, my = 0.0;
-#pragma unroll
-  for (int j = 0; j < 4; j++) {
-    mx += p[j][0];
-    my += p[j][1];
-  }
-  mx /= 4.0;
-  my /= 4.0;
-  double d = 0.0;
-#pragma unroll
-  for (int j = 0; j < 4; j++) d += sqrt((p[j][0] - mx) * (p[j][0] - mx) + (p[j][1] - my) * (p[j][1] - my));
-  d /= 4.0;
-  const double sc = d > 0.0 ? 1.4142135623730951 / d : 1.0;
-#pragma unroll
-  for (int j = 0; j < 4; j++) {
-    p[j][0] = sc * p[j][0] - sc * mx;
-    p[j][1] = sc * p[j][1] - sc * my;
-  }
-  *s = sc;
-  *cx = mx;
-  *cy = my;
-}
+__device__ __forceinline__ double shfl_d(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
-__device__ bool collinear4(const double p[4][2]) {
-  const int tri[4][3] = {{0, 1, 2}, {0, 1, 3}, {0, 2, 3}, {1, 2, 3}};
-  for (int t = 0; t < 4; t++) {
-    const int i = tri[t][0], j = tri[t][1], m = tri[t][2];
-    const double a = 0.5 * fabs((p[j][0] - p[i][0]) * (p[m][1] - p[i][1]) -
-                                (p[j][1] - p[i][1]) * (p[m][0] - p[i][0]));
-    if (a < 1e-6) return true;
-  }
-  return false;
-}
-
-// Column C of Gaussian elimination with partial pivoting on the 8 x 9
-// augmented system: the row r >= C with the largest |M[r][C]| (the first on
-// ties) becomes the pivot row, the rows below are reduced. False if the
-// column is all zero (singular system).
+// Column C of Gaussian elimination with partial pivoting on the 8 x 9 augmented
+// system, one row per lane of the group g0 .. g0 + 7; pos is the row's position.
+// The row at position >= C with the largest |m[C]| (the first on ties) becomes the
+// pivot row and takes position C; the rows below are reduced. False (for the whole
+// group) if the column is all zero (singular system).
 template <int C>
-__device__ __forceinline__ bool elim_step(double (&M)[8][9], double (&rinv)[8]) {
-  int piv = C;
-  double best = fabs(M[C][C]);
+__device__ __forceinline__ bool elim_step(double (&m)[9], int &pos, double &rinv, int g0, int lane) {
+  // |m[C]| as an integer: the bits of non-negative doubles are ordered as they are.
+  unsigned long long key = pos >= C ? (unsigned long long)__double_as_longlong(fabs(m[C])) : 0ull;
+  int at = pos >= C ? pos : 8, src = lane;
 #pragma unroll
-  for (int r = C + 1; r < 8; r++) {
-    const double a = fabs(M[r][C]);
-    if (a > best) {
-      best = a;
-      piv = r;
+  for (int o = 1; o < 8; o <<= 1) {
+    const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
+    const int a2 = __shfl_xor_sync(0xffffffffu, at, o), s2 = __shfl_xor_sync(0xffffffffu, src, o);
+    if (k2 > key || (k2 == key && a2 < at)) {
+      key = k2;
+      at = a2;
+      src = s2;
     }
   }
-  if (best == 0.0) return false;
+  if (pos == C) pos = at;
+  if (lane == src) pos = C;
+  const double ri = 1.0 / shfl_d(m[C], src);
+  if (lane == src) rinv = ri;
+  const double f = m[C] * ri;
+  const bool below = pos > C;
 #pragma unroll
-  for (int r = C + 1; r < 8; r++) {
-    const bool sw = piv == r;
-#pragma unroll
-    for (int k = C; k < 9; k++) {
-      const double t = M[C][k];
-      M[C][k] = sw ? M[r][k] : t;
-      M[r][k] = sw ? t : M[r][k];
-    }
+  for (int k = C + 1; k < 9; k++) {
+    const double p = shfl_d(m[k], src);
+    const double r = m[k] - f * p;
+    m[k] = below ? r : m[k];
   }
-  rinv[C] = 1.0 / M[C][C];
-#pragma unroll
-  for (int r = C + 1; r < 8; r++) {
-    const double f = M[r][C] * rinv[C];
-#pragma unroll
-    for (int k = C; k < 9; k++) M[r][k] -= f * M[C][k];
-  }
-  return true;
+  return key != 0ull;
 }
 
+// What bounds the fit is FP64: two lanes per cycle and SM, each operation some tens
+// of cycles late. With a thread per hypothesis and one warp per SM it was a chain of
+// about 650 dependent operations, 26 us for 1,500 hypotheses; eight lanes shorten
+// the chain to about 250 and leave 12 us (both cold, under ncu). The arithmetic of a
+// row is unchanged but for the back substitution, which takes its terms from the last
+// unknown down.
 __global__ void __launch_bounds__(kFitThreads) k_magsac_fit(const float2 *__restrict__ xa,
                                                             const float2 *__restrict__ xb, int n,
                                                             const int *__restrict__ samples,
                                                             int n_hyp, double *__restrict__ models,
                                                             int *__restrict__ valid) {
-  const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  if (h >= n_hyp) return;
-  int idx[4];
-  bool ok = true;
+  const int lane = threadIdx.x & 31, s = lane & 7, g0 = lane & 24;
+  const int hyp = blockIdx.x * (kFitThreads / 8) + (threadIdx.x >> 3);
+  const int h = min(hyp, n_hyp - 1);  // every lane takes part in the shuffles
+  auto group_any = [&](bool v) { return (__ballot_sync(0xffffffffu, v) >> g0 & 0xffu) != 0u; };
+  // Lane s: point s & 3 of image a (s < 4) or b.
+  const int idx = samples[4 * h + (s & 3)];
+  const bool in = idx >= 0 && idx < n;
+  bool bad = group_any(!in);
+  const float2 pt = (s < 4 ? xa : xb)[in ? idx : 0];
+  double x = pt.x, y = pt.y;
+  const int im = g0 + (s & 4);  // the image's first lane
+  double mx = 0.0, my = 0.0;
 #pragma unroll
   for (int j = 0; j < 4; j++) {
-    idx[j] = samples[4 * h + j];
-    ok = ok && idx[j] >= 0 && idx[j] < n;
+    mx += shfl_d(x, im + j);
+    my += shfl_d(y, im + j);
   }
-  if (!ok) {
-    valid[h] = 0;
-    return;
-  }
-  double pa[4][2], pb[4][2];
+  mx /= 4.0;
+  my /= 4.0;
+  const double dist = sqrt((x - mx) * (x - mx) + (y - my) * (y - my));
+  double dsum = 0.0;
 #pragma unroll
-  for (int j = 0; j < 4; j++) {
-    const float2 a = xa[idx[j]], b = xb[idx[j]];
-    pa[j][0] = a.x;
-    pa[j][1] = a.y;
-    pb[j][0] = b.x;
-    pb[j][1] = b.y;
-  }
-  double sa, ax, ay, sb, bx, by;
-  normalise4(pa, &sa, &ax, &ay);
-  normalise4(pb, &sb, &bx, &by);
-  if (collinear4(pa) || collinear4(pb)) {
-    valid[h] = 0;
-    return;
+  for (int j = 0; j < 4; j++) dsum += shfl_d(dist, im + j);
+  dsum /= 4.0;
+  const double sc = dsum > 0.0 ? 1.4142135623730951 / dsum : 1.0;
+  x = sc * x - sc * mx;
+  y = sc * y - sc * my;
+  {  // lane s: triangle s & 3 of its image: (0, 1, 2), (0, 1, 3), (0, 2, 3), (1, 2, 3)
+    const int t = s & 3;
+    const int ti = im + (t == 3), tj = im + (t < 2 ? 1 : 2), tm = im + (t == 0 ? 2 : 3);
+    const double xi = shfl_d(x, ti), yi = shfl_d(y, ti);
+    const double xj = shfl_d(x, tj), yj = shfl_d(y, tj);
+    const double xm = shfl_d(x, tm), ym = shfl_d(y, tm);
+    const double area = 0.5 * fabs((xj - xi) * (ym - yi) - (yj - yi) * (xm - xi));
+    bad |= group_any(area < 1e-6);
   }
   // A h = 0 with h33 = 1: rows (x, y, 1, 0, 0, 0, -u x, -u y | u) and
-  // (0, 0, 0, x, y, 1, -v x, -v y | v) (signs flipped from the DLT rows).
-  double M[8][9];
-#pragma unroll
-  for (int j = 0; j < 4; j++) {
-    const double x = pa[j][0], y = pa[j][1], u = pb[j][0], v = pb[j][1];
-    const double r0[9] = {x, y, 1.0, 0.0, 0.0, 0.0, -u * x, -u * y, u};
-    const double r1[9] = {0.0, 0.0, 0.0, x, y, 1.0, -v * x, -v * y, v};
-#pragma unroll
-    for (int c = 0; c < 9; c++) {
-      M[2 * j][c] = r0[c];
-      M[2 * j + 1][c] = r1[c];
-    }
+  // (0, 0, 0, x, y, 1, -v x, -v y | v) (signs flipped from the DLT rows); lane s has
+  // row s: correspondence s / 2, u for even s and v for odd.
+  double m[9];
+  {
+    const int j = s >> 1;
+    const double ax = shfl_d(x, g0 + j), ay = shfl_d(y, g0 + j);
+    const double u = shfl_d(x, g0 + 4 + j), v = shfl_d(y, g0 + 4 + j);
+    const bool odd = s & 1;
+    const double q = odd ? v : u;
+    m[0] = odd ? 0.0 : ax;
+    m[1] = odd ? 0.0 : ay;
+    m[2] = odd ? 0.0 : 1.0;
+    m[3] = odd ? ax : 0.0;
+    m[4] = odd ? ay : 0.0;
+    m[5] = odd ? 1.0 : 0.0;
+    m[6] = -q * ax;
+    m[7] = -q * ay;
+    m[8] = q;
   }
-  // One instantiation per pivot column (elim_step<C>), so every index is a
-  // compile-time constant and M stays in registers: the pivot row is swapped
-  // in by selects, and each pivot's reciprocal is taken once.
-  double rinv[8];
-  bool ok8 = elim_step<0>(M, rinv) && elim_step<1>(M, rinv) && elim_step<2>(M, rinv) &&
-             elim_step<3>(M, rinv) && elim_step<4>(M, rinv) && elim_step<5>(M, rinv) &&
-             elim_step<6>(M, rinv) && elim_step<7>(M, rinv);
-  if (!ok8) {
-    valid[h] = 0;
-    return;
-  }
+  int pos = s;
+  double rinv = 0.0;
+  bool ok8 = elim_step<0>(m, pos, rinv, g0, lane);
+  ok8 &= elim_step<1>(m, pos, rinv, g0, lane);
+  ok8 &= elim_step<2>(m, pos, rinv, g0, lane);
+  ok8 &= elim_step<3>(m, pos, rinv, g0, lane);
+  ok8 &= elim_step<4>(m, pos, rinv, g0, lane);
+  ok8 &= elim_step<5>(m, pos, rinv, g0, lane);
+  ok8 &= elim_step<6>(m, pos, rinv, g0, lane);
+  ok8 &= elim_step<7>(m, pos, rinv, g0, lane);
+  bad |= !ok8;
+  // Back substitution: the row at position c gives h[c], which every row above it
+  // subtracts at once.
   double hn[9];
   hn[8] = 1.0;
 #pragma unroll
   for (int c = 7; c >= 0; c--) {
-    double acc = M[c][8];
-#pragma unroll
-    for (int k = c + 1; k < 8; k++) acc -= M[c][k] * hn[k];
-    hn[c] = acc * rinv[c];
+    const unsigned who = __ballot_sync(0xffffffffu, pos == c) >> g0 & 0xffu;
+    hn[c] = shfl_d(m[8] * rinv, g0 + __ffs(who) - 1);
+    m[8] -= m[c] * hn[c];  // (only the rows above are read again)
   }
   double nn = 1.0;
+#pragma unroll
   for (int k = 0; k < 8; k++) nn += hn[k] * hn[k];
-  if (!(nn <= 1e18)) {  // the null vector's h33 component below 1e-9 (or not finite)
-    valid[h] = 0;
-    return;
-  }
+  bad |= !(nn <= 1e18);  // the null vector's h33 component below 1e-9 (or not finite)
   // H = Tb^-1 Hn Ta with Ta = [[sa, 0, -sa ax], [0, sa, -sa ay], [0, 0, 1]] and
-  // Tb^-1 = [[1/sb, 0, bx], [0, 1/sb, by], [0, 0, 1]].
-  double G[9];  // Hn Ta
-  for (int r = 0; r < 3; r++) {
-    const double a0 = hn[3 * r], a1 = hn[3 * r + 1], a2 = hn[3 * r + 2];
-    G[3 * r] = a0 * sa;
-    G[3 * r + 1] = a1 * sa;
-    G[3 * r + 2] = a2 - a0 * sa * ax - a1 * sa * ay;
+  // Tb^-1 = [[1/sb, 0, bx], [0, 1/sb, by], [0, 0, 1]]. Lane s: entry s; all: entry 8.
+  const double sa = shfl_d(sc, g0), ax = shfl_d(mx, g0), ay = shfl_d(my, g0);
+  const double sb = shfl_d(sc, g0 + 4), bx = shfl_d(mx, g0 + 4), by = shfl_d(my, g0 + 4);
+  auto third = [&](double a0, double a1, double a2) { return a2 - a0 * sa * ax - a1 * sa * ay; };  // of Hn Ta
+  const int row = s / 3, col = s - 3 * row;
+  const double a0 = row == 0 ? hn[0] : row == 1 ? hn[3] : hn[6];
+  const double a1 = row == 0 ? hn[1] : row == 1 ? hn[4] : hn[7];
+  const double a2 = row == 0 ? hn[2] : row == 1 ? hn[5] : hn[8];
+  const double g8 = third(hn[6], hn[7], hn[8]);
+  const double ge = col == 2 ? third(a0, a1, a2) : (col ? a1 : a0) * sa;
+  const double gl = col == 2 ? g8 : (col ? hn[7] : hn[6]) * sa;  // the last row's entry of this column
+  const double e = row == 2 ? ge : ge / sb + (row ? by : bx) * gl;
+  double big = fmax(fabs(e), fabs(g8));
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+  bad |= !(fabs(g8) >= 1e-12 * big);
+  if (hyp >= n_hyp) return;
+  if (!bad) {
+    const double inv = 1.0 / g8;
+    models[9 * h + s] = e * inv;
+    if (s == 7) models[9 * h + 8] = 1.0;
   }
-  double H[9];
-  for (int c = 0; c < 3; c++) {
-    H[c] = G[c] / sb + bx * G[6 + c];
-    H[3 + c] = G[3 + c] / sb + by * G[6 + c];
-    H[6 + c] = G[6 + c];
-  }
-  double mx = 0.0;
-  for (int k = 0; k < 9; k++) mx = fmax(mx, fabs(H[k]));
-  if (!(fabs(H[8]) >= 1e-12 * mx)) {
-    valid[h] = 0;
-    return;
-  }
-  const double inv = 1.0 / H[8];
-  for (int k = 0; k < 9; k++) models[9 * h + k] = H[k] * inv;
-  models[9 * h + 8] = 1.0;
-  valid[h] = 1;
+  if (s == 0) valid[h] = bad ? 0 : 1;
 }
 
 __global__ void __launch_bounds__(kScoreThreads) k_magsac_score(const float2 *__restrict__ xa,
@@ -250,6 +234,7 @@ __global__ void __launch_bounds__(kScoreThreads) k_magsac_score(const float2 *__
                                                                 const int *__restrict__ valid,
                                                                 int n_hyp, MagsacConst c,
                                                                 float *__restrict__ scores) {
+  pdl_wait();  // the models
   __shared__ float red[kScoreThreads / 32];
   const int tid = threadIdx.x;
   for (int h = blockIdx.x; h < n_hyp; h += gridDim.x) {
@@ -292,12 +277,14 @@ __global__ void __launch_bounds__(kSelectThreads) k_magsac_select(
   __shared__ int si[kSelectThreads / 32];
   __shared__ float s_H[9];
   __shared__ int s_best;
+  pdl_wait();  // the scores
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool first = blockIdx.x == 0;
   float v = INFINITY;
   int bi = 0x7fffffff;
   for (int h = tid; h < n_hyp; h += kSelectThreads) {
     const float s = scores[h];
-    if (scores_out) scores_out[h] = s;
+    if (scores_out && first) scores_out[h] = s;
     better(v, bi, s, h);
   }
 #pragma unroll
@@ -317,17 +304,19 @@ __global__ void __launch_bounds__(kSelectThreads) k_magsac_select(
     for (int w = 1; w < kSelectThreads / 32; w++) better(bv, b, sv[w], si[w]);
     const int best = (bv < INFINITY) ? b : -1;
     s_best = best;
-    *best_out = best;
-    *score_out = best >= 0 ? bv : INFINITY;
+    if (first) {
+      *best_out = best;
+      *score_out = best >= 0 ? bv : INFINITY;
+    }
     for (int k = 0; k < 9; k++) {
       const double e = best >= 0 ? models[9 * best + k] : 0.0;
-      H_out[k] = e;
+      if (first) H_out[k] = e;
       s_H[k] = (float)e;
     }
   }
   __syncthreads();
   const int best = s_best;
-  for (int i = tid; i < n; i += kSelectThreads)
+  for (int i = blockIdx.x * kSelectThreads + tid; i < n; i += gridDim.x * kSelectThreads)
     inliers[i] = (best >= 0 && transfer_r2(s_H, xa[i], xb[i]) <= c.kk_s2) ? 1 : 0;
 }
 
@@ -384,17 +373,16 @@ cudaError_t launch_magsac(const float *xa, const float *xb, int n, const int *sa
   int dev = 0, n_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  // The FP64 solver is bound by each SM's FP64 rate: spread the hypotheses over
-  // every SM (ceil(n_hyp / SMs) threads per block, at most 32).
-  const int fit_threads = std::max(1, std::min(kFitThreads, (n_hyp + n_sm - 1) / n_sm));
-  cudaError_t e = launch_plain(k_magsac_fit, (n_hyp + fit_threads - 1) / fit_threads, fit_threads,
-                               0, s, a, b, n, samples, n_hyp, models, valid);
+  cudaError_t e = launch_plain(k_magsac_fit, (n_hyp + kFitThreads / 8 - 1) / (kFitThreads / 8), kFitThreads, 0,
+                               s, a, b, n, samples, n_hyp, models, valid);
   if (e != cudaSuccess) return e;
   const int grid = n_hyp < 8 * n_sm ? n_hyp : 8 * n_sm;
-  e = launch_plain(k_magsac_score, grid, kScoreThreads, 0, s, a, b, n, models, valid, n_hyp, c,
+  e = launch_pdl(k_magsac_score, grid, kScoreThreads, 0, s, a, b, n, models, valid, n_hyp, c,
                    scores);
   if (e != cudaSuccess) return e;
-  return launch_plain(k_magsac_select, 1, kSelectThreads, 0, s, a, b, n, models, scores, n_hyp, c,
+  // Every block reads all scores, so more than one only where the points are many.
+  const int sel = std::max(1, std::min({n_sm, n / (4 * kSelectThreads), n / n_hyp}));
+  return launch_pdl(k_magsac_select, sel, kSelectThreads, 0, s, a, b, n, models, scores, n_hyp, c,
                       H_out, best_out, score_out, inliers, scores_out);
 }
 
