@@ -51,11 +51,23 @@ __device__ __forceinline__ LevelView<HF> level_at(const float *L, long long lofs
 // octaves (fp16 storage mode) and the level type is chosen per keypoint.
 constexpr int kOriWarps = 8;
 
+// 1 / x to about one unit in the last place, for finite x >= FLT_MIN.
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // Nearest-bin vote of one gradient: weight wgt into bin floor(36 theta / 2 pi
-// + 1/2) of lane's column.
-__device__ __forceinline__ void ori_vote(float (*hist)[32], int lane, float dx, float dy,
-                                         float wgt) {
-  const float mag = sqrtf(dx * dx + dy * dy);
+// + 1/2) of lane's column. The bin comes from an odd polynomial in min / max of
+// |dx| and |dy| (its relative minimax fit to atan on [0, 1], in bins, exchange
+// algorithm: 2e-5 bins off at most with its FP32 evaluation) where that puts theta
+// at least kVoteMargin bins from a boundary; the rest, one sample in 2,500, and all
+// gradients with |dx| = |dy|, take atan2f, whose own error is below 1e-5 bins. So
+// every vote is the one that atan2f gives, at about 25 instructions fewer.
+constexpr float kVoteMargin = 2e-4f;
+
+__device__ __noinline__ int ori_bin_exact(float dx, float dy) {
   float th = atan2f(dy, dx);
   if (th < 0.f) th += kTwoPi;
   int bin = (int)floorf(th * ((float)kOriBins / kTwoPi) + 0.5f);
@@ -67,7 +79,37 @@ __device__ __forceinline__ void ori_vote(float (*hist)[32], int lane, float dx, 
     const int qd = dy > 0.f ? (dx > 0.f ? 0 : 1) : (dx < 0.f ? 2 : 3);
     bin = (kOriBins * (2 * qd + 1) + 4) / 8 % kOriBins;
   }
-  hist[bin][lane] += wgt * mag;
+  return bin;
+}
+
+__device__ __forceinline__ int ori_bin(float dx, float dy) {
+  const float ax = fabsf(dx), ay = fabsf(dy);
+  const float t = fminf(ax, ay) * rcp_approx(fmaxf(fmaxf(ax, ay), 1.17549435e-38f));
+  const float u = t * t;
+  float r = -0.0772374049f;
+  r = fmaf(r, u, 0.329320759f);
+  r = fmaf(r, u, -0.694648683f);
+  r = fmaf(r, u, 1.12092124f);
+  r = fmaf(r, u, -1.90791845f);
+  r = fmaf(r, u, 5.72955275f);
+  r *= t;
+  r = ay > ax ? 9.f - r : r;
+  r = dx < 0.f ? 18.f - r : r;
+  r = dy < 0.f ? 36.f - r : r;  // theta in bins, [0, 36]
+  // Nearest integer and distance from it: adding 1.5 * 2^23 rounds to an integer,
+  // which is then in the low bits of the sum.
+  const float m = r + 12582912.f;
+  int bin = __float_as_int(m) & 63;
+  bin = bin == kOriBins ? 0 : bin;
+  // (not <, so that NaN goes the exact way too)
+  if (!(fabsf(r - (m - 12582912.f)) < 0.5f - kVoteMargin)) bin = ori_bin_exact(dx, dy);
+  return bin;
+}
+
+__device__ __forceinline__ void ori_vote(float (*hist)[32], int lane, float dx, float dy,
+                                         float wgt) {
+  const float mag = sqrtf(dx * dx + dy * dy);
+  hist[ori_bin(dx, dy)][lane] += wgt * mag;
 }
 
 // The window's samples, lane l taking samples l, l + 32, l + 64, ... in that
@@ -507,9 +549,42 @@ constexpr int kDescCols = 16;
 // Floats of one warp's histogram block: 128 bins x 16 columns.
 constexpr int kDescWarpFloats = kDescLen * kDescCols;
 
+// atan2(y, x) in eighths of a turn, [0, 8]. The polynomial is the relative minimax
+// fit to atan on [0, 1] (exchange algorithm, 1.5e-8; 1.5e-7 evaluated in FP32), so
+// that with the quotient's rounding the result is as close as atan2f's (3 ulp) times
+// 8 / 2 pi: the descriptors' distance from 64 bits is unchanged.
+__device__ __forceinline__ float atan2_eighths(float y, float x) {
+  const float ax = fabsf(x), ay = fabsf(y);
+  const float t = fminf(ax, ay) * rcp_approx(fmaxf(fmaxf(ax, ay), 1.17549435e-38f));
+  const float u = t * t;
+  float r = 0.00362859224f;
+  r = fmaf(r, u, -0.0204592142f);
+  r = fmaf(r, u, 0.0543565303f);
+  r = fmaf(r, u, -0.0955476463f);
+  r = fmaf(r, u, 0.135484576f);
+  r = fmaf(r, u, -0.180846423f);
+  r = fmaf(r, u, 0.254553944f);
+  r = fmaf(r, u, -0.424409866f);
+  r = fmaf(r, u, 1.27323949f);
+  r *= t;
+  r = ay > ax ? 2.f - r : r;
+  r = x < 0.f ? 4.f - r : r;
+  return y < 0.f ? 8.f - r : r;
+}
+
+// floor(x) as a float and (low bits) an integer, for |x| < 2^21, by rounding x - 1/2
+// to the nearest integer: 1.5 * 2^23 is added and subtracted. At an integer x it may
+// give x - 1, with a fraction of 1 instead of 0: the same linear split over two bins.
+__device__ __forceinline__ float split_floor(float x, int *i) {
+  const float m = (x - 0.5f) + 12582912.f;
+  *i = __float_as_int(m) - 0x4b400000;
+  return m - 12582912.f;
+}
+
 // The trilinear targets of one gradient sample at bin coordinates (rx, ry)
 // from the keypoint, (u, v) = (rx, ry) + 3/2: weight m * exp(-(rx^2 + ry^2) /
-// 8), orientation relative to th. Cells outside the 4 x 4 grid get -1.
+// 8), orientation relative to th8 (eighths of a turn). Cells outside the 4 x 4 grid
+// get -1.
 struct Vote {
   int cell[4];    // (v * 4 + u) * 8 * kDescCols (the cell's first histogram word), or -1
   float w[4];     // spatial weights times the magnitude-Gaussian weight
@@ -521,26 +596,22 @@ struct Vote {
 // four of its cells are then -1, so that the commit skips it without a
 // branch around this function.
 __device__ __forceinline__ void desc_targets(Vote &v, float rx, float ry, float gx, float gy,
-                                             float th, bool ok = true) {
+                                             float th8, bool ok = true) {
   const float u = rx + 1.5f, vv0 = ry + 1.5f;
   const float mag = sqrtf(gx * gx + gy * gy);
-  float phi = atan2f(gy, gx) - th;
-  if (phi < 0.f) phi += kTwoPi;
-  if (phi < 0.f) phi += kTwoPi;
-  if (phi >= kTwoPi) phi -= kTwoPi;
-  const float ob = phi * (8.0f / kTwoPi);
+  float ob = atan2_eighths(gy, gx) - th8;
+  ob = ob < 0.f ? ob + 8.f : ob;
   const float wt = mag * expf(-(rx * rx + ry * ry) * 0.125f);
-  const float u0f = floorf(u), v0f = floorf(vv0), o0f = floorf(ob);
-  const float fu = u - u0f, fv = vv0 - v0f, f1 = ob - o0f;
-  const int u0 = (int)u0f, v0 = (int)v0f, o0 = (int)o0f & 7, o1 = (o0 + 1) & 7;
-  const bool even0 = (o0 & 1) == 0;
-  v.oe = (even0 ? o0 : o1) * kDescCols;
-  v.oo = (even0 ? o1 : o0) * kDescCols;
-  v.fe = even0 ? 1.f - f1 : f1;
-  v.fo = even0 ? f1 : 1.f - f1;
-  // u0, v0 lie in [-1, 3] (u, v in (-1, 4)): cell u0 + du exists iff u0 >= 0
-  // (du = 0) or u0 <= 2 (du = 1), and the same for v.
-  const bool uok[2] = {ok && u0 >= 0, ok && u0 <= 2}, vok[2] = {v0 >= 0, v0 <= 2};
+  int u0, v0, o0;
+  const float fu = u - split_floor(u, &u0), fv = vv0 - split_floor(vv0, &v0);
+  const float f1 = ob - split_floor(ob, &o0);
+  const bool odd0 = o0 & 1;
+  v.oe = ((o0 + 1) & 6) * kDescCols;
+  v.oo = (o0 & 7 | 1) * kDescCols;
+  v.fe = odd0 ? f1 : 1.f - f1;
+  v.fo = odd0 ? 1.f - f1 : f1;
+  const bool uok[2] = {ok && (unsigned)u0 < 4u, ok && (unsigned)(u0 + 1) < 4u};
+  const bool vok[2] = {(unsigned)v0 < 4u, (unsigned)(v0 + 1) < 4u};
   const int c00 = (v0 * 4 + u0) * 8;
 #pragma unroll
   for (int dv = 0; dv < 2; dv++) {
@@ -580,7 +651,7 @@ __constant__ float kDspScale[5] = {0.5f, 0.70710678118654752f, 1.0f, 1.414213562
 template <bool HF>
 __device__ __forceinline__ void desc_sweep(const Desc *__restrict__ d, const RefRec &r,
                                            const OctDev &od, const float *L, long long lofs,
-                                           float wbin, float inv_w, float th, float st,
+                                           float wbin, float inv_w, float th8, float st,
                                            float ct, int R, float *hist, int lane, int warp,
                                            int (*s_lo)[32], int (*s_pre)[33]) {
   const int tid = threadIdx.x;
@@ -677,9 +748,9 @@ __device__ __forceinline__ void desc_sweep(const Desc *__restrict__ d, const Ref
           const float ga = lv[oa + 1] - lv[oa - 1], ha = lv[oa + pitch] - lv[oa - pitch];
           const float gb = lv[ob + 1] - lv[ob - 1], hb = lv[ob + pitch] - lv[ob - pitch];
           Vote vt;
-          desc_targets(vt, rxa, rya, ga, ha, th, oka);
+          desc_targets(vt, rxa, rya, ga, ha, th8, oka);
           desc_commit(hist, lane, vt);
-          desc_targets(vt, rxb, ryb, gb, hb, th, okb);
+          desc_targets(vt, rxb, ryb, gb, hb, th8, okb);
           desc_commit(hist, lane, vt);
         }
         __syncwarp();  // the next round rewrites this warp's interval table
@@ -716,7 +787,7 @@ __device__ __forceinline__ void desc_sweep(const Desc *__restrict__ d, const Ref
                            fy * (gx1 * at(p2) + fx * at(p2 + 1));
           const float ym = gy1 * (gx1 * at(pm) + fx * at(pm + 1)) +
                            fy * (gx1 * at(p) + fx * at(p + 1));
-          desc_targets(vt, rx, ry, xp - xm, yp - ym, th);
+          desc_targets(vt, rx, ry, xp - xm, yp - ym, th8);
           desc_commit(hist, lane, vt);
         }
       }
@@ -808,7 +879,7 @@ __global__ void __launch_bounds__(kKpWarps * 32, 6) k_descriptor(const Desc *__r
       for (int k = lane; k < kDescLen * kDescCols / 4; k += 32) h4[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncwarp();
-    desc_sweep<PART == 2>(d, r, od, L, lofs, wbin, inv_w, th, st, ct, R, hist, lane, warp, s_lo, s_pre);
+    desc_sweep<PART == 2>(d, r, od, L, lofs, wbin, inv_w, angle * (8.0f / 360.0f), st, ct, R, hist, lane, warp, s_lo, s_pre);
     __syncthreads();
     // Bin tid: per warp, the 16 columns starting at column (tid / 2) % 16 (with
     // the layout [bin][16], the 32 threads of a warp then read 32 distinct

@@ -315,7 +315,9 @@ __global__ void __launch_bounds__(kThreads) k_bm_compact(const Desc *__restrict_
   __shared__ int s_val;
   constexpr int WPT = kChunk / kThreads;  // words per thread
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int n = d->n_img, C = d->n_bm_chunks, G = gridDim.x, g = blockIdx.x;
+  // (no more blocks than chunks: a short list's look-back is short)
+  const int n = d->n_img, C = d->n_bm_chunks, G = min((int)gridDim.x, C), g = blockIdx.x;
+  if (g >= G) return;
   const LookbackCfg cfg{d->lb_epoch, d->lb_spins, d->lb_hold, d->lb_err};
   const int ca = (int)((long long)C * g / G), cb = (int)((long long)C * (g + 1) / G);
   const int kept = min(cb - ca, kMaxCh);
