@@ -7,6 +7,8 @@
 // touched by one thread at a time, in an order fixed by the code); the
 // columns are then summed bin by bin in a fixed order. No atomics are used
 // anywhere, so outputs are bitwise reproducible.
+#include <type_traits>
+
 #include "scan.cuh"
 #include "sift_dev.cuh"
 
@@ -51,10 +53,10 @@ __device__ __forceinline__ LevelView<HF> level_at(const float *L, long long lofs
 // octaves (fp16 storage mode) and the level type is chosen per keypoint.
 constexpr int kOriWarps = 8;
 
-// 1 / x to about one unit in the last place, for finite x >= FLT_MIN.
+// 1 / x to about one unit in the last place, for x in [FLT_MIN, 2^126] (0 above).
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 
@@ -83,8 +85,8 @@ __device__ __noinline__ int ori_bin_exact(float dx, float dy) {
 }
 
 __device__ __forceinline__ int ori_bin(float dx, float dy) {
-  const float ax = fabsf(dx), ay = fabsf(dy);
-  const float t = fminf(ax, ay) * rcp_approx(fmaxf(fmaxf(ax, ay), 1.17549435e-38f));
+  const float ax = fabsf(dx), ay = fabsf(dy), am = fmaxf(fmaxf(ax, ay), 1.17549435e-38f);
+  const float t = fminf(ax, ay) * rcp_approx(am);
   const float u = t * t;
   float r = -0.0772374049f;
   r = fmaf(r, u, 0.329320759f);
@@ -101,8 +103,8 @@ __device__ __forceinline__ int ori_bin(float dx, float dy) {
   const float m = r + 12582912.f;
   int bin = __float_as_int(m) & 63;
   bin = bin == kOriBins ? 0 : bin;
-  // (not <, so that NaN goes the exact way too)
-  if (!(fabsf(r - (m - 12582912.f)) < 0.5f - kVoteMargin)) bin = ori_bin_exact(dx, dy);
+  // (so that NaN and reciprocals out of range go the exact way too)
+  if (!(fabsf(r - (m - 12582912.f)) < 0.5f - kVoteMargin && am < 1e37f)) bin = ori_bin_exact(dx, dy);
   return bin;
 }
 
@@ -115,52 +117,58 @@ __device__ __forceinline__ void ori_vote(float (*hist)[32], int lane, float dx, 
 // The window's samples, lane l taking samples l, l + 32, l + 64, ... in that
 // order, three per step: the twelve loads of a step are issued before any of
 // its votes, so that more loads are in flight per warp.
-template <bool HF>
+// IN: the whole window and its neighbours lie inside the level (nearly always).
+template <bool HF, bool IN>
 __device__ __forceinline__ void ori_sweep(const float *__restrict__ L, long long lofs, int pitch,
                                           int H, int W, int x0, int y0, int R, float ninv,
                                           float (*hist)[32], int lane) {
   const LevelView<HF> v = level_at<HF>(L, lofs, pitch, x0, y0);
+  const LevelView<HF> up = level_at<HF>(L, lofs, pitch, x0, y0 - 1), dn = level_at<HF>(L, lofs, pitch, x0, y0 + 1);
   const int side = 2 * R + 1, nsamp = side * side;
-  // Sample q = jj * side + c; advancing q by 32 adds dr rows and dc columns.
+  // Sample q = (j + R) * side + (i + R), off = j * pitch + i; advancing q by 32 adds
+  // dr rows and dc columns.
   const int dr = 32 / side, dc = 32 - dr * side;
-  int jj = lane / side, c = lane - jj * side;
+  const int doff = dr * pitch + dc, wrap = pitch - side;
+  const int j0 = lane / side;
+  int j = j0 - R, i = lane - j0 * side - R, off = j * pitch + i;
   auto advance = [&]() {
-    c += dc;
-    jj += dr;
-    if (c >= side) {
-      c -= side;
-      jj++;
+    i += dc;
+    j += dr;
+    off += doff;
+    if (i > R) {
+      i -= side;
+      j++;
+      off += wrap;
     }
-  };
-  // Inside the window with a full 3 x 3 neighbourhood in the level.
-  auto inside = [&](int q, int i, int j) {
-    const int px = x0 + i, py = y0 + j;
-    return q < nsamp && px >= 1 && px <= W - 2 && py >= 1 && py <= H - 2;
   };
   // Without branches: a sample outside the window or the image reads the
   // keypoint's own pixel neighbourhood (always inside: keypoints keep the
   // border) and votes with weight 0, which leaves its bin unchanged.
   constexpr int NS = 3;
   for (int q = lane; q < nsamp; q += 32 * NS) {
-    int ii[NS], jv[NS], off[NS];
+    float r2[NS];
+    int at[NS];
     bool ok[NS];
 #pragma unroll
     for (int k = 0; k < NS; k++) {
-      ii[k] = c - R;
-      jv[k] = jj - R;
+      r2[k] = (float)(i * i + j * j);
+      ok[k] = q + 32 * k < nsamp;
+      if (!IN) {
+        const int px = x0 + i, py = y0 + j;
+        ok[k] = ok[k] && px >= 1 && px <= W - 2 && py >= 1 && py <= H - 2;
+      }
+      at[k] = ok[k] ? off : 0;
       advance();
-      ok[k] = inside(q + 32 * k, ii[k], jv[k]);
-      off[k] = ok[k] ? jv[k] * pitch + ii[k] : 0;
     }
     float gx[NS], gy[NS];
 #pragma unroll
     for (int k = 0; k < NS; k++) {
-      gx[k] = v[off[k] + 1] - v[off[k] - 1];
-      gy[k] = v[off[k] + pitch] - v[off[k] - pitch];
+      gx[k] = v[at[k] + 1] - v[at[k] - 1];
+      gy[k] = dn[at[k]] - up[at[k]];
     }
 #pragma unroll
     for (int k = 0; k < NS; k++) {
-      const float w = expf((float)(ii[k] * ii[k] + jv[k] * jv[k]) * ninv);
+      const float w = expf(r2[k] * ninv);
       ori_vote(hist, lane, gx[k], gy[k], ok[k] ? w : 0.f);
     }
   }
@@ -214,10 +222,15 @@ __global__ void __launch_bounds__(kOriWarps * 32, 4) k_orientation(const Desc *_
       const float ninv = -1.0f / (2.0f * sw * sw);
 #pragma unroll 4
       for (int k = 0; k < kOriBins; k++) hist[k][lane] = 0.f;
-      if (MIXED && od.half != 0)
-        ori_sweep<true>(L, lofs, od.pitch, od.H, od.W, r.x, r.y, R, ninv, hist, lane);
-      else
-        ori_sweep<false>(L, lofs, od.pitch, od.H, od.W, r.x, r.y, R, ninv, hist, lane);
+      const bool whole = r.x > R && r.x + R <= od.W - 2 && r.y > R && r.y + R <= od.H - 2;
+      auto sweep = [&](auto hf, auto in) {
+        ori_sweep<decltype(hf)::value, decltype(in)::value>(L, lofs, od.pitch, od.H, od.W, r.x, r.y, R, ninv,
+                                                            hist, lane);
+      };
+      using T = std::true_type;
+      using F = std::false_type;
+      if (MIXED && od.half != 0) whole ? sweep(T(), T()) : sweep(T(), F());
+      else whole ? sweep(F(), T()) : sweep(F(), F());
       __syncwarp();
       // Bin k: the 32 columns in the order k, k + 1, ... (mod 32); the rotated
       // start puts the lanes on distinct banks.
@@ -583,18 +596,18 @@ __device__ __forceinline__ float split_floor(float x, int *i) {
 
 // The trilinear targets of one gradient sample at bin coordinates (rx, ry)
 // from the keypoint, (u, v) = (rx, ry) + 3/2: weight m * exp(-(rx^2 + ry^2) /
-// 8), orientation relative to th8 (eighths of a turn). Cells outside the 4 x 4 grid
-// get -1.
+// 8), orientation relative to th8 (eighths of a turn).
 struct Vote {
-  int cell[4];    // (v * 4 + u) * 8 * kDescCols (the cell's first histogram word), or -1
-  float w[4];     // spatial weights times the magnitude-Gaussian weight
-  int oe, oo;     // the even and the odd orientation bin, times kDescCols
-  float fe, fo;   // their orientation weights
+  int cell;        // ((v0 * 4 + u0) * 8) * kDescCols, the first cell's histogram word
+  bool ok[4];      // whether cells (v0, u0), (v0, u0 + 1), (v0 + 1, u0), (v0 + 1, u0 + 1) exist
+  float w[4];      // spatial weights times the magnitude-Gaussian weight
+  int oe, oo;      // the even and the odd orientation bin, times kDescCols
+  float fe, fo;    // their orientation weights
 };
 
-// ok false: the lane has no sample (its coordinates may lie anywhere); all
-// four of its cells are then -1, so that the commit skips it without a
-// branch around this function.
+// ok false: the lane has no sample (its coordinates may lie anywhere); none of
+// its four cells exists, so that the commit skips it without a branch around
+// this function.
 __device__ __forceinline__ void desc_targets(Vote &v, float rx, float ry, float gx, float gy,
                                              float th8, bool ok = true) {
   const float u = rx + 1.5f, vv0 = ry + 1.5f;
@@ -609,36 +622,40 @@ __device__ __forceinline__ void desc_targets(Vote &v, float rx, float ry, float 
   v.oe = ((o0 + 1) & 6) * kDescCols;
   v.oo = (o0 & 7 | 1) * kDescCols;
   v.fe = odd0 ? f1 : 1.f - f1;
-  v.fo = odd0 ? 1.f - f1 : f1;
-  const bool uok[2] = {ok && (unsigned)u0 < 4u, ok && (unsigned)(u0 + 1) < 4u};
-  const bool vok[2] = {(unsigned)v0 < 4u, (unsigned)(v0 + 1) < 4u};
-  const int c00 = (v0 * 4 + u0) * 8;
-#pragma unroll
-  for (int dv = 0; dv < 2; dv++) {
-    const float wv = wt * (dv ? fv : 1.f - fv);
-#pragma unroll
-    for (int du = 0; du < 2; du++) {
-      const float wu = du ? fu : 1.f - fu;
-      v.cell[dv * 2 + du] = (uok[du] && vok[dv]) ? (c00 + (dv * 4 + du) * 8) * kDescCols : -1;
-      v.w[dv * 2 + du] = wv * wu;
-    }
-  }
+  v.fo = 1.f - v.fe;
+  v.cell = (v0 * 4 + u0) * (8 * kDescCols);
+  const bool ua = (unsigned)u0 < 4u, ub = (unsigned)(u0 + 1) < 4u;
+  const bool va = ok && (unsigned)v0 < 4u, vb = ok && (unsigned)(v0 + 1) < 4u;
+  v.ok[0] = va && ua;
+  v.ok[1] = va && ub;
+  v.ok[2] = vb && ua;
+  v.ok[3] = vb && ub;
+  const float w1 = wt * fv, w0 = wt - w1;
+  v.w[1] = w0 * fu;
+  v.w[0] = w0 - v.w[1];
+  v.w[3] = w1 * fu;
+  v.w[2] = w1 - v.w[3];
 }
 
 // Add the votes of the warp's lanes to the warp's columns in the two passes
 // described above; a vote without a target (a cell outside the grid) is
-// skipped. Every lane of the warp must call it.
+// skipped. A lane's four cells are different words at fixed distances: their
+// loads are issued together. Every lane of the warp must call it.
 __device__ __forceinline__ void desc_commit(float *hist, int lane, const Vote &v) {
-  float *col = hist + (lane & (kDescCols - 1));
+  constexpr int kStep[4] = {0, 8 * kDescCols, 32 * kDescCols, 40 * kDescCols};
+  float *col = hist + (lane & (kDescCols - 1)) + v.cell;
   const bool upper = lane >= 16;
 #pragma unroll
   for (int pass = 0; pass < 2; pass++) {
     const bool even = (pass == 0) != upper;
-    const int o = even ? v.oe : v.oo;
+    float *c = col + (even ? v.oe : v.oo);
     const float f = even ? v.fe : v.fo;
+    float h[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) h[k] = v.ok[k] ? c[kStep[k]] : 0.f;
 #pragma unroll
     for (int k = 0; k < 4; k++)
-      if (v.cell[k] >= 0) col[v.cell[k] + o] += v.w[k] * f;
+      if (v.ok[k]) c[kStep[k]] = fmaf(v.w[k], f, h[k]);
     __syncwarp();
   }
 }
@@ -715,7 +732,7 @@ __device__ __forceinline__ void desc_sweep(const Desc *__restrict__ d, const Ref
         const int tot = __shfl_sync(0xffffffffu, pre, 31);
         pre -= len;
         int *wlo = s_lo[warp], *wpre = s_pre[warp];
-        wlo[lane] = a0;
+        wlo[lane] = a0 - pre;  // sample q of the list is column q + wlo[row]
         wpre[lane] = pre;
         if (lane == 31) wpre[32] = tot;
         __syncwarp();
@@ -727,7 +744,7 @@ __device__ __forceinline__ void desc_sweep(const Desc *__restrict__ d, const Ref
           if (q >= tot) return false;
           while (wpre[row + 1] <= q) row++;
           const int jy = jlo + warp + kKpWarps * (rb + row);
-          const int i = wlo[row] + (q - wpre[row]);
+          const int i = wlo[row] + q;
           const float ox = (float)i - r.dx, oy = (float)jy - r.dy;
           rx = (ct * ox + st * oy) * inv_w;
           ry = (-st * ox + ct * oy) * inv_w;
@@ -769,8 +786,7 @@ __device__ __forceinline__ void desc_sweep(const Desc *__restrict__ d, const Ref
           const bool ok = !(x0 < 1 || x0 > od.W - 3 || y0 < 1 || y0 > od.H - 3);
           Vote vt;
           if (!ok) {  // (1024 samples per scale: the trip count is warp-uniform)
-#pragma unroll
-            for (int k = 0; k < 4; k++) vt.cell[k] = -1;
+            vt = Vote{};
             desc_commit(hist, lane, vt);
             continue;
           }
