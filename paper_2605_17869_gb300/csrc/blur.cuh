@@ -119,16 +119,39 @@ constexpr int item_rows(int th) { return th / 4; }
 // MODE 1: octave 0 level 0 from the input image.
 // MODE 3: level 1 of octave `oct` > 0 from its level 0, decimated on the fly
 //         from level S of octave oct - 1; level 0 itself is stored on the way.
-struct TileGeo {
+struct alignas(16) TileGeo {
   const float *src;  // staging source: level lvl_out - 1 (MODE 0), the input (1),
                      // level S of the previous octave (3)
   float *out;        // level lvl_out of the tile's octave
-  float *out0;       // level 0 of the tile's octave (MODE 3 stores it)
-  int spitch;        // source pitch (elements)
   int pitch, H, W;   // the octave's pitch and size
   int vec;           // 16-byte aligned source rows
   int x0, y0;
+  int spitch;        // source pitch (elements)
+  int pad;
+  float *out0;       // level 0 of the tile's octave (MODE 3 stores it)
 };
+// A tile's geometry from shared memory by 16-byte loads, once per tile (field by
+// field, for the tile and for the next one's copies, it was a fifth of the R = 5
+// kernel's shared-memory accesses).
+template <int MODE> __device__ __forceinline__ TileGeo load_geo(const TileGeo *p) {
+  const int4 *q = reinterpret_cast<const int4 *>(p);
+  const int4 a = q[0], b = q[1], c = q[2];
+  auto ptr = [](int lo, int hi) {
+    return reinterpret_cast<float *>((unsigned long long)(unsigned)lo | (unsigned long long)(unsigned)hi << 32);
+  };
+  TileGeo g;
+  g.src = ptr(a.x, a.y);
+  g.out = ptr(a.z, a.w);
+  g.pitch = b.x;
+  g.H = b.y;
+  g.W = b.z;
+  g.vec = MODE == 0 ? 1 : b.w;
+  g.x0 = c.x;
+  g.y0 = c.y;
+  g.spitch = MODE == 0 ? b.x : c.z;
+  g.out0 = MODE == 3 ? p->out0 : nullptr;
+  return g;
+}
 
 // Geometry of flattened tile t. Image b's octaves sit at fixed slots
 // oct[b * kMaxOct + o], so no ImgDev read is needed for pyramid levels.
@@ -366,8 +389,9 @@ __device__ __forceinline__ void row_pass_store(const float *s_v, float *out, int
   const int hl = lane >> 4, l = lane & 15;
   const int x = x0 + 8 * l;
   const bool xok = x < pitch;  // pitches are multiples of 32: all eight or none
+  constexpr int IT = TH / (2 * kWarps);  // rows per half-warp
 #pragma unroll 1
-  for (int v = 2 * warp + hl; v < TH; v += 2 * kWarps) {
+  for (int it = 0, v = 2 * warp + hl; it < IT; it++, v += 2 * kWarps) {
     const float4 *s4 = reinterpret_cast<const float4 *>(s_v + v * kSinW) + l;
     float in[S::NV * 4];
 #pragma unroll
@@ -455,18 +479,22 @@ __global__ void __launch_bounds__(kThreads, TH == 20 ? 4 : 3)
   if (threadIdx.x < 32) fill_chunk(0);
   __syncthreads();
   pdl_wait();  // the source level is the previous kernel's output
-  issue_stage<R, TH, MODE, ST>(geo[0], s_in);
+  TileGeo g = load_geo<MODE>(&geo[0]);
+  issue_stage<R, TH, MODE, ST>(g, s_in);
   for (int k = 0; k < n_mine; k++) {
     if (k + 1 == n_mine) pdl_trigger();  // successors launch during this block's last tile
-    const TileGeo &g = geo[k & (2 * kGeoChunk - 1)];
-    const TileGeo &gn = geo[(k + 1) & (2 * kGeoChunk - 1)];
     cp_async_wait_all();
     __syncthreads();
     if (MODE == 3) store_level0<R, TH, ST != 0, KIND>(s_in, g.out0, g.pitch, g.H, g.x0, g.y0);
     col_pass<R, TH, KIND>(s_in, s_v, tp);
     __syncthreads();
-    if (k + 1 < n_mine) issue_stage<R, TH, MODE, ST>(gn, s_in);
+    TileGeo gn = g;
+    if (k + 1 < n_mine) {
+      gn = load_geo<MODE>(&geo[(k + 1) & (2 * kGeoChunk - 1)]);
+      issue_stage<R, TH, MODE, ST>(gn, s_in);
+    }
     row_pass_store<R, TH, ST != 0>(s_v, g.out, g.pitch, g.H, g.x0, g.y0, tp);
+    g = gn;
     if (threadIdx.x < 32 && (k & (kGeoChunk - 1)) == kGeoChunk / 2)
       fill_chunk(k / kGeoChunk + 1);
     // No barrier here: the barrier after the next copy-wait orders every
