@@ -123,7 +123,11 @@ __device__ __forceinline__ void ext_test(const ExtRow<S> &P, const ExtRow<S> &C,
   for (int s = 0; s < S; s++) gate |= (fabsf(C.c[s][0]) > thr0) | (fabsf(C.c[s][1]) > thr1);
   unsigned lo = 0u, hi = 0u;
   if (yin && __any_sync(0xffffffffu, gate)) {
-    bool ok[S][2], any = false;
+    // First the extrema that may be shared with a neighbour: |c| above the gate and
+    // c at least (at most) the maximum (minimum) over the 27 values, five
+    // instructions per value; a row of the strip that has one (about one in six)
+    // is then tested strictly, which takes nine.
+    bool any = false;
 #pragma unroll
     for (int k = 0; k < 2; k++) {
       float vx[S + 2], vn[S + 2];
@@ -135,15 +139,26 @@ __device__ __forceinline__ void ext_test(const ExtRow<S> &P, const ExtRow<S> &C,
 #pragma unroll
       for (int s = 1; s <= S; s++) {
         const float c = C.c[s - 1][k];
-        const float lf = k ? C.c[s - 1][0] : C.l[s - 1], rt = k ? C.r[s - 1] : C.c[s - 1][1];
-        const float mx = fmaxf(max3f(vx[s - 1], vx[s + 1], lf), max3f(P.hx[s][k], N.hx[s][k], rt));
-        const float mn = fminf(min3f(vn[s - 1], vn[s + 1], lf), min3f(P.hn[s][k], N.hn[s][k], rt));
-        ok[s - 1][k] = ((c > mx) | (c < mn)) & (fabsf(c) > (k ? thr1 : thr0));
-        any |= ok[s - 1][k];
+        any |= ((c >= max3f(vx[s - 1], vx[s], vx[s + 1])) | (c <= min3f(vn[s - 1], vn[s], vn[s + 1]))) &
+               (fabsf(c) > (k ? thr1 : thr0));
       }
     }
     if (__any_sync(0xffffffffu, any)) {
-unsigned m0 = 0u, m1 = 0u;  // lane s: layer s + 1 at the lanes' first / second columns
+      bool ok[S][2];
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+#pragma unroll
+        for (int s = 1; s <= S; s++) {
+          const float c = C.c[s - 1][k];
+          const float lf = k ? C.c[s - 1][0] : C.l[s - 1], rt = k ? C.r[s - 1] : C.c[s - 1][1];
+          float mx = max3f(max3f(P.hx[s][k], N.hx[s][k], lf), rt, max3f(P.hx[s - 1][k], C.hx[s - 1][k], N.hx[s - 1][k]));
+          float mn = min3f(min3f(P.hn[s][k], N.hn[s][k], lf), rt, min3f(P.hn[s - 1][k], C.hn[s - 1][k], N.hn[s - 1][k]));
+          mx = fmaxf(mx, max3f(P.hx[s + 1][k], C.hx[s + 1][k], N.hx[s + 1][k]));
+          mn = fminf(mn, min3f(P.hn[s + 1][k], C.hn[s + 1][k], N.hn[s + 1][k]));
+          ok[s - 1][k] = ((c > mx) | (c < mn)) & (fabsf(c) > (k ? thr1 : thr0));
+        }
+      }
+      unsigned m0 = 0u, m1 = 0u;  // lane s: layer s + 1 at the lanes' first / second columns
 #pragma unroll
       for (int s = 0; s < S; s++) {
         const unsigned b0 = __ballot_sync(0xffffffffu, ok[s][0]), b1 = __ballot_sync(0xffffffffu, ok[s][1]);
@@ -169,14 +184,14 @@ unsigned m0 = 0u, m1 = 0u;  // lane s: layer s + 1 at the lanes' first / second 
 // The candidate decisions are exact comparisons of the same FP32 values, so they do
 // not depend on the tiling. Bitmap words are written by ballots; no atomics.
 // Two columns per lane share the copies, the loop, two of four shuffles per layer
-// and the middle values of the three-column extrema: 3.5 warp instructions per
-// tested pixel column against 4.9 with one column. What bounds it is the ALU pipe
-// (66%: three-input extrema and comparisons) together with HBM (52%, every level
-// value read once) at 16 warps per SM, which 128 registers allow (12 warps at 150:
-// 2 percent more per call on the 64-image batch); rings of 4 and 8 rows were no
-// faster than 3. Octave 0 of half that batch: 170 us before, 165 now; all scans of
-// four 1024 x 768 images with five layers, whose strips of one column per lane left
-// 8 warps per SM: 333 -> 286 us per call.
+// and the middle values of the three-column extrema. What bounds the scan is the
+// ALU pipe (66%: three-input extrema and comparisons) together with HBM (52%, every
+// level value read once) at 16 warps per SM, which 128 registers allow (12 warps at
+// 150: 2 percent more per call on the 64-image batch); rings of 4 and 8 rows were no
+// faster than 3. All scans of the 64-image batch: 545 us with one column per lane
+// (4.9 warp instructions per pixel and warp row), 480 with two (3.5), 439 with the
+// two-stage test of ext_test; of four 1024 x 768 images with five layers, whose
+// one-column strips left 8 warps per SM, 333 -> 276 us per call.
 // HALF: the octave's levels are binary16 (fp16 storage mode): a lane's two columns
 // are one 32-bit word, widened when the row is read.
 template <int S, bool HALF>
