@@ -372,21 +372,21 @@ def profiled_classes(torch, ex, step, flush, reps):
 def _traffic_per_launch(px_step, blur_n):
     """DRAM bytes of an average level-blur launch of this workload: the per-pixel
     DRAM traffic of a captured level-blur launch (profiles/blur_level_traffic.json)
-    times the pixels an average launch processes; only while pyramid.cu is the
+    times the pixels an average launch processes; only while blur.cuh is the
     source the counters were read from."""
     tpath = os.path.join(ROOT, "profiles", "blur_level_traffic.json")
     if not os.path.exists(tpath) or not blur_n:
         return None
     with open(tpath) as f:
         tj = json.load(f)
-    src = open(os.path.join(ROOT, "paper_2605_17869_gb300", "csrc", "pyramid.cu"), "rb").read()
-    if tj.get("pyramid_cu_sha256") != hashlib.sha256(src).hexdigest():
+    src = open(os.path.join(ROOT, "paper_2605_17869_gb300", "csrc", "blur.cuh"), "rb").read()
+    if tj.get("blur_cuh_sha256") != hashlib.sha256(src).hexdigest():
         return None
     return int(tj["dram_bytes_per_px"] * px_step / blur_n)
 
 
 def _is_default_tuning(js):
-    """Whether a tuning JSON is the defaults (32-row tiles, occupancy-maximum
+    """Whether a tuning JSON is the defaults (row class 32, occupancy-maximum
     grids, a batch split over two lanes): a tuned time then differs from the
     untuned one by noise only."""
     t = json.loads(js)
@@ -528,7 +528,7 @@ def gpu_arm(args, rank, world, pool, batch):
     if args.tuning:
         ex.set_tuning(args.tuning)
     else:
-        # The defaults first (32-row tiles, occupancy-maximum grids), then the
+        # The defaults first (row class 32, occupancy-maximum grids), then the
         # batch autotuner on this very batch; the timed steps use its choice.
         n_def = max(10, args.steps // 4)
         t_def, _ = queued_steps(torch, step, n_def, args.warmup, stream)
@@ -938,7 +938,7 @@ def main():
     ap.add_argument("--images", type=int, default=N_IMAGES,
                     help=f"images per batch (default {N_IMAGES}; the first n of the batch)")
     ap.add_argument("--serving-requests", type=int, default=SERVING_REQUESTS)
-    ap.add_argument("--tuning", default="", help='fixed tiles, e.g. {"blur_tile_rows": [32,...]}')
+    ap.add_argument("--tuning", default="", help='fixed row classes, e.g. {"blur_tile_rows": [32,...]}')
     ap.add_argument("--tuning-cache", default="",
                     help="tuning cache file for the batch autotuner (default: none, always search)")
     args = ap.parse_args()

@@ -316,9 +316,11 @@ sift_status sift_last_launch_count(sift_handle *h, int *kernels);
  * which CTA computes what, never the arithmetic, so every tuning gives
  * bit-identical outputs. Its JSON form, every key optional:
  *   {"blur_tile_rows": [[r_1, ..., r_{S+2}], ...],  per octave, one entry per
- *                                                   level blur; 32 or 64 rows
- *                                                   (binary16 levels of the
- *                                                   fp16 mode always use 32);
+ *                                                   level blur; row class 32
+ *                                                   (20-row tiles) or 64 (40-
+ *                                                   row tiles; binary16 levels
+ *                                                   of the fp16 mode always
+ *                                                   use 32);
  *                                                   a flat list sets octave 0
  *    "blur_ctas_per_sm": [c_0, c_1, ...],           level blurs, per octave
  *    "extrema_ctas_per_sm": c, "orientation_ctas_per_sm": c,
@@ -333,7 +335,7 @@ sift_status sift_last_launch_count(sift_handle *h, int *kernels);
  * string, an unknown key or a value out of range); sift_get_tuning writes the
  * full tuning (SIFT_E_INVALID if len is too small).
  *
- * sift_autotune: for each level blur of octave 0, time 32- and 64-row tiles
+ * sift_autotune: for each level blur of octave 0, time the row classes 32 and 64
  * on a synthetic H x W pyramid on `stream` and keep the faster. */
 sift_status sift_autotune(sift_handle *h, int H, int W, void *stream);
 sift_status sift_get_tuning(sift_handle *h, char *json, size_t len);
@@ -343,7 +345,7 @@ sift_status sift_set_tuning(sift_handle *h, const char *json);
  * images), plus from_cache (host, may be NULL) set to 1 when the tuning came
  * from the cache. Coordinate descent over whole extraction steps of this
  * batch on `stream` (each run as sift_extract_batch runs it, lanes included),
- * from the defaults: 64-row tiles per level of the three
+ * from the defaults: row class 64 per level of the three
  * largest octaves, then fewer resident CTAs per SM for their level blurs and
  * for the extrema, orientation, descriptor and compaction grids, then 1 to 4
  * lanes (batch_lanes); a change is kept only if the step gets at least 1%

@@ -12,10 +12,10 @@
 //  * TH = 20, V = 5: the column pass is 80 pairs x 4 row blocks, one item per
 //    thread, and the row pass 10 pairs of rows, one per warp, so that neither pass
 //    leaves warps waiting at the two barriers of a tile. What bounds the kernel is
-//    neither HBM (24-46% of its bandwidth) nor the FMA pipe (43% at R = 5, 59% at R
-//    = 13) nor shared memory (50-60%) but the waits at barriers and on loads, so
-//    four or more blocks per SM matter more than the halo rows that a short tile
-//    stages again (from L2). Measured on the 64-image batch, 1024 x 768 x 4 images
+//    the L1 and shared-memory path (70-72% busy) with the waits at barriers and on
+//    loads, not HBM (28-43% of its bandwidth) or the FMA pipe (41% at R = 5, 56% at
+//    R = 13), so four blocks per SM matter more than the halo rows that a short tile
+//    stages again (from L2). Measured when the tile was chosen, on the 64-image batch, 1024 x 768 x 4 images
 //    at five scales per octave, and one 640 x 480 image (us per call): TH = 20: 2367
 //    / 334 / 135; TH = 30: 2407 / 339 / 145; TH = 40 with 640 threads: 2433 / 360 /
 //    148, with 320 threads and V = 10: 2425 / 407 / 147. A ring of rows marched down
@@ -27,7 +27,7 @@
 //    from the odd ones, so that lanes two groups apart read without conflicts.
 //
 // Every output pixel is the same fixed-order chain of FP32 operations whatever
-// the step or strip: out(y, x) = sum_i w_i * c_i with c_i = sum_j w_j * in(y - R
+// the tile height: out(y, x) = sum_i w_i * c_i with c_i = sum_j w_j * in(y - R
 // + j, x - R + i), each c_i summed over j ascending and the outer sum split into
 // two ascending chains of alternate taps whose grouping depends only on the
 // parity of x - R (row_pass_store). Results therefore do not depend on the

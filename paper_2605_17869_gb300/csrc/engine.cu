@@ -835,8 +835,8 @@ sift_status Engine::autotune(int H, int W, cudaStream_t s) {
   // Time the whole pyramid stage (all octaves, as the pipeline runs it), not
   // one level in isolation: a level's tile height also changes how the level
   // overlaps its neighbours and how warm L2 is for them. Coordinate descent
-  // from 32-row tiles everywhere in octave 0; a level switches to 64 rows only
-  // if the stage gets at least 1% faster.
+  // from the smaller tiles everywhere in octave 0; a level switches to the larger
+  // ones only if the stage gets at least 1% faster.
   auto time_stage = [&]() -> float {
     for (int w = 0; w < 2; w++) enqueue_all(s, M, modes, nullptr, false, true);
     cudaEventRecord(a, s);
@@ -920,9 +920,9 @@ sift_status Engine::autotune_batch(int n, const ImgIn *imgs, cudaStream_t s, con
     M = std::max(M, octave_sizes(imgs[i].H, imgs[i].W, hs, ws));
   }
   // Coordinate descent over whole extraction steps of the caller's batch,
-  // starting from the defaults (32-row tiles, occupancy-maximum grids): a
+  // starting from the defaults (the smaller tiles, occupancy-maximum grids): a
   // candidate replaces the incumbent only if the step gets at least 1% faster.
-  // Searched, in order: 64-row tiles per FP32 level of the three largest
+  // Searched, in order: the larger tiles per FP32 level of the three largest
   // octaves (smaller octaves have too few tiles to fill the GPU), fewer
   // resident blur CTAs per SM for those octaves, then fewer extrema,
   // orientation and descriptor CTAs per SM (down to half the maximum).

@@ -8,7 +8,7 @@
 //    "blur_ctas_per_sm": [c_0, c_1, ...],            per octave
 //    "extrema_ctas_per_sm": c, "orientation_ctas_per_sm": c,
 //    "descriptor_ctas_per_sm": c, "compaction_ctas_per_sm": c, "batch_lanes": 1 .. 4}
-// r is 32 or 64; c is 0 (the occupancy maximum) or 1..64 (capped by the
+// r is a row class, 32 (20-row tiles) or 64 (40-row tiles); c is 0 (the occupancy maximum) or 1..64 (capped by the
 // occupancy maximum at launch).
 //
 // Cache file: {"version": 1, "entries": {"<signature>": <tuning JSON>, ...}}.
