@@ -381,6 +381,8 @@ cudaError_t launch_magsac(const float *xa, const float *xb, int n, const int *sa
                    scores);
   if (e != cudaSuccess) return e;
   // Every block reads all scores, so more than one only where the points are many.
+  // One block against this many (us, cold): 8,192 points and 1,500 hypotheses 12.8
+  // against 8.9, 20,011 and 500 23.8 against 9.8, 65,536 and 500 66 against 8.5.
   const int sel = std::max(1, std::min({n_sm, n / (4 * kSelectThreads), n / n_hyp}));
   return launch_pdl(k_magsac_select, sel, kSelectThreads, 0, s, a, b, n, models, scores, n_hyp, c,
                       H_out, best_out, score_out, inliers, scores_out);

@@ -126,7 +126,7 @@ struct Desc {
   // after the other, so a small octave's scan takes as long as its strips are).
   int ext_rows[kMaxOct];
   int tile_pre[TK_COUNT][kMaxOct][kMaxImg + 1];
-  // Base-blur work of the images with up = 0 (steps, or tiles at radius 0) / 1 (tiles).
+  // Base-blur tiles of the images with up = 0 / 1.
   int base_pre[2][kMaxImg + 1];
   int bmc_pre[kMaxImg + 1];
   int cc_pre[kMaxImg + 1];
