@@ -403,11 +403,7 @@ sift_status sift_build_pyramid(sift_handle *h, const float *img_dev, int H, int 
   cudaStream_t s = (cudaStream_t)stream;
   h->split_batch = false;
   h->n_parts = 0;
-  st = h->eng->run_pyramid(in, s);
-  if (st != SIFT_OK) return pass(h, st);
-  const cudaError_t e = sift::launch_export(h->eng->device_desc(), out_dev, h->eng->sm_count(), s);
-  if (e != cudaSuccess) return fail(h, SIFT_E_CUDA, cudaGetErrorString(e));
-  return SIFT_OK;
+  return pass(h, h->eng->run_pyramid(in, s, out_dev));
 }
 
 sift_status sift_set_profiling(sift_handle *h, int enable) {

@@ -703,7 +703,7 @@ sift_status Engine::run(int n, const ImgIn *imgs, cudaStream_t s) {
   return SIFT_OK;
 }
 
-sift_status Engine::run_pyramid(const ImgIn &img, cudaStream_t s) {
+sift_status Engine::run_pyramid(const ImgIn &img, cudaStream_t s, float *out) {
   sift_status st = init();
   if (st != SIFT_OK) return st;
   const int slot = (ring_ + 1) % kRing;
@@ -729,7 +729,11 @@ sift_status Engine::run_pyramid(const ImgIn &img, cudaStream_t s) {
   if (st == SIFT_OK) st = upload(hd, bytes, s);
   if (st != SIFT_OK) return st;
   cudaError_t e = cudaGraphLaunch(exec, s);
-  if (e == cudaSuccess) e = cudaEventRecord(done_, s);
+  // done_ comes after the copy, which reads the device descriptor and the
+  // workspace: the next call may overwrite or free both once done_ has passed.
+  if (e == cudaSuccess && out) e = launch_export(ddesc_, out, n_sm_, s);
+  const cudaError_t er = cudaEventRecord(done_, s);
+  if (e == cudaSuccess) e = er;
   if (e != cudaSuccess) {
     err = std::string("pyramid launch failed: ") + cudaGetErrorString(e);
     return SIFT_E_CUDA;
@@ -825,7 +829,7 @@ sift_status Engine::autotune(int H, int W, cudaStream_t s) {
   in.H = H;
   in.W = W;
   in.pitch = W;
-  st = run_pyramid(in, s);
+  st = run_pyramid(in, s, nullptr);
   int hs[kMaxOct], ws[kMaxOct];
   const int M = octave_sizes(H, W, hs, ws);
   const int modes = magnify(H, W) ? 2 : 1;

@@ -75,7 +75,8 @@ class Engine {
   // Queue the extraction of n <= kMaxImg images on stream s.
   sift_status run(int n, const ImgIn *imgs, cudaStream_t s);
   // Queue the pyramid stage only (for export); one image.
-  sift_status run_pyramid(const ImgIn &img, cudaStream_t s);
+  // out: dense planes of the pyramid (launch_export), or null for none.
+  sift_status run_pyramid(const ImgIn &img, cudaStream_t s, float *out);
   // Whether an H x W input gets the 2x magnified first octave: upsample on
   // and at most upsample_max_px input pixels (0: no limit).
   bool magnify(int H, int W) const;
