@@ -44,8 +44,10 @@ __device__ __forceinline__ void stage_upsampled(const float *__restrict__ src, i
 }
 
 // The same output from scalar operations, for the generic kernel: row points
-// at the output's first tap column s, odd tells the parity of s.
+// at the output's first tap column s, odd tells the parity of s. Radius 0 has one
+// tap only (the chains below take at least three).
 __device__ __forceinline__ float row_tap_sum(const float *row, bool odd, int R, const float *w) {
+  if (R == 0) return __fmul_rn(w[0], row[0]);
   float ax, ay;
   if (!odd) {
     ax = __fmul_rn(w[0], row[0]);
