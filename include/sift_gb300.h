@@ -199,8 +199,8 @@ sift_status sift_extract_noalloc(const sift_params *p, const float *img_dev, int
  *   out_match_a: device, n_a ints: j for a kept pair (i, j), else -1; -2 in
  *   every entry if a bounded device wait gave up (the run is not valid).
  * Asynchronous on `stream`; the handle keeps a small workspace that grows with
- * n_a + n_b. Errors: SIFT_E_INVALID for a null pointer, n_a or n_b outside
- * [0, 65536] or ratio outside (0, 1]; SIFT_E_OOM / SIFT_E_CUDA. With fewer
+ * n_a + n_b. Errors: SIFT_E_INVALID for a null or misaligned pointer, n_a or n_b
+ * outside [0, 65536] or ratio outside (0, 1]; SIFT_E_OOM / SIFT_E_CUDA. With fewer
  * than two descriptors on either side no pair is kept. */
 sift_status sift_match(sift_handle *h, const float *desc_a, int n_a, const float *desc_b, int n_b,
                        float ratio, void *stream, int *out_match_a);

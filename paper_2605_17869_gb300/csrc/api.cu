@@ -203,6 +203,9 @@ sift_status sift_match(sift_handle *h, const float *desc_a, int n_a, const float
   if ((n_a > 0 && (!desc_a || !out_match_a)) || (n_b > 0 && !desc_b))
     return fail(h, SIFT_E_INVALID, "null pointer argument");
   if (n_a == 0) return SIFT_OK;
+  // The conversion reads rows by 16-byte loads; an empty set is not read.
+  if ((reinterpret_cast<uintptr_t>(desc_a) & 15) || (n_b > 0 && (reinterpret_cast<uintptr_t>(desc_b) & 15)))
+    return fail(h, SIFT_E_INVALID, "descriptor sets must be 16-byte aligned");
   const cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (!h->match_attr) {
     if (sift::match_set_attributes() != cudaSuccess) return fail(h, SIFT_E_CUDA, "matcher attributes");
