@@ -214,8 +214,9 @@ sift_status sift_match(sift_handle *h, const float *desc_a, int n_a, const float
  * response, then N int32 each of octave, layer (540 bytes per keypoint; the
  * per-image counts split it). dst_dev: device, 16-byte aligned, at least
  * 540 x images x max_kpts bytes. Asynchronous. Errors: SIFT_E_INVALID for a
- * null or misaligned dst, a short dst, no extraction yet, or a last batch of
- * more than 128 images; SIFT_E_CUDA. */
+ * null or misaligned dst, a short dst, no extraction yet, a last batch of more
+ * than 128 images, or a descriptor buffer of the last call that is not 16-byte
+ * aligned; SIFT_E_CUDA. */
 sift_status sift_pack_outputs(sift_handle *h, void *stream, void *dst_dev, size_t dst_bytes);
 
 /* GPU MAGSAC++ homography verification (§3.6 "GPU MAGSAC++"): the best of

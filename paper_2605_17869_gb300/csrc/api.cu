@@ -246,6 +246,10 @@ sift_status sift_pack_outputs(sift_handle *h, void *stream, void *dst_dev, size_
       return fail(h, SIFT_E_INVALID, "the last call on this handle was not an extraction");
     src.d[k] = e->device_desc();
     n_img += (size_t)e->last_n;
+    // The copy reads descriptor rows by 16-byte loads (an extraction takes any buffer of floats).
+    for (int b = 0; b < e->last_n; b++)
+      if (reinterpret_cast<uintptr_t>(e->host_desc().img[b].odesc) & 15)
+        return fail(h, SIFT_E_INVALID, "the last call's descriptor buffers are not all 16-byte aligned");
   }
   const size_t need = n_img * h->eng->params().max_kpts * (sift::kDescLen * sizeof(float) + 7 * 4);
   if (dst_bytes < need) return fail(h, SIFT_E_INVALID, "dst smaller than last_n * max_kpts * 540 bytes");

@@ -95,7 +95,7 @@ class Engine {
   bool addressable(int H, int W) const;
   // Workspace bytes a batch needs (serving admission).
   size_t workspace_bytes(int n, const int *H, const int *W) const;
-  // Device-side per-image geometry of the last run (valid until the next run).
+  // Host copy of the last run's descriptor (valid until the next run).
   const Desc &host_desc() const { return *hdesc_[ring_last_]; }
   const WsLayout &layout() const { return lay_; }
   // Device descriptor of the last run (valid on its stream until the next run).
