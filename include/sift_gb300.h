@@ -354,7 +354,7 @@ sift_status sift_set_tuning(sift_handle *h, const char *json);
  * the output buffers hold this batch's results (a run with that tuning;
  * identical to sift_extract_batch's). Synchronises `stream` while timing.
  * With a tuning cache set (sift_set_tuning_cache), the batch's signature
- * (device and sift_batch_signature) is looked up first: a hit applies the
+ * (device, kernels and sift_batch_signature) is looked up first: a hit applies the
  * stored tuning and runs the batch once, without timing; a miss tunes and then
  * stores the result. SIFT_E_INVALID also for an unreadable cache file or an
  * invalid entry, and when the cache cannot be written. */
@@ -373,7 +373,9 @@ sift_status sift_set_tuning_cache(sift_handle *h, const char *path);
 /* Host only. The batch part of a tuning-cache signature: every parameter that
  * changes the work, the image count, total pixels, longest side and a 64-bit
  * FNV-1a hash of the sorted (H, W) list (a reordered batch has the same
- * signature). sift_autotune_batch prefixes "sm<major><minor>x<SMs>;".
+ * signature). sift_autotune_batch prefixes "sm<major><minor>x<SMs>;k<n>;", n the
+ * generation of the library's kernels (2): a tuning that was found with other
+ * kernels is not applied.
  * SIFT_E_INVALID on invalid parameters or sizes, or if len is too small. */
 sift_status sift_batch_signature(const sift_params *p, int n, const int *H, const int *W,
                                  char *out, size_t len);

@@ -879,7 +879,8 @@ std::string Engine::device_key() const {
   int ma = 0, mi = 0;
   cudaDeviceGetAttribute(&ma, cudaDevAttrComputeCapabilityMajor, dev_);
   cudaDeviceGetAttribute(&mi, cudaDevAttrComputeCapabilityMinor, dev_);
-  return "sm" + std::to_string(ma) + std::to_string(mi) + "x" + std::to_string(n_sm_);
+  return "sm" + std::to_string(ma) + std::to_string(mi) + "x" + std::to_string(n_sm_) + ";k" +
+         std::to_string(kTuningKernels);
 }
 
 float Engine::time_steps(const Tuning &t, const StepFn &step, cudaStream_t s, sift_status *st) {

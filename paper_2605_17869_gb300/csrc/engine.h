@@ -53,6 +53,11 @@ constexpr int kMaxLanes = 4;  // largest batch_lanes
 void lookback_config(int *spins, int *hold);
 
 // Host-only tuning helpers (tuning.cu).
+// Part of every tuning-cache key, raised whenever the kernels that were timed or
+// what a tuning's numbers mean change, so that a cache file's earlier entries are
+// not applied (they would be shapes that nothing measured). 2: row classes 32 and 64
+// are tiles of 20 and 40 rows; entries without a number were tuned for 32 and 64 rows.
+constexpr int kTuningKernels = 2;
 Tuning default_tuning();
 std::string tuning_json(const Tuning &t, int n_scales);
 bool parse_tuning(const char *json, int n_scales, const Tuning &base, Tuning *out,
@@ -124,7 +129,8 @@ class Engine {
   using StepFn = std::function<sift_status()>;
   sift_status autotune_batch(int n, const ImgIn *imgs, cudaStream_t s,
                              const StepFn &step = StepFn());
-  // "sm<major><minor>x<SMs>": the device part of a tuning-cache key.
+  // "sm<major><minor>x<SMs>;k<kTuningKernels>": the part of a tuning-cache key
+  // that the batch does not decide.
   std::string device_key() const;
   int level_radius(int l) const { return lvl_R_[l]; }
 
