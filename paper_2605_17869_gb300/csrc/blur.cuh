@@ -1,6 +1,7 @@
 // Separable Gaussian level blur (§3.2, "GPU Pipeline Stages"), 4-sigma
-// truncation, reflect-101 borders: the kernel template, instantiated per radius
-// by the blur_r*.cu units and launched by pyramid.cu.
+// truncation, reflect-101 borders: the kernel template, instantiated and launched by
+// pyramid.cu (radii of the default scale space), blur_rest.cu and blur_rest64.cu (the
+// others).
 //
 // One launch computes one pyramid level for every image of the batch: a
 // persistent grid of ten-warp blocks walks a flattened queue of 128 x TH output
@@ -509,25 +510,24 @@ struct BlurFn {
   const void *fn;
   int smem;
 };
-template <int R> BlurFn blur_instance(int variant) {
 #define SIFT_BLUR_FN(TH, MODE, ST) \
   BlurFn{reinterpret_cast<const void *>(k_blur<R, TH, MODE, ST>), blur_smem<R, TH, MODE, ST>()}
+template <int R> BlurFn blur_instance(int variant) {  // 20-row tiles
   switch (variant) {
     case BV_LVL: return SIFT_BLUR_FN(20, 0, 0);
     case BV_DEC: return SIFT_BLUR_FN(20, 3, 0);
     case BV_LVL_H16: return SIFT_BLUR_FN(20, 0, 2);
     case BV_DEC_R16: return SIFT_BLUR_FN(20, 3, 1);
     case BV_DEC_H16: return SIFT_BLUR_FN(20, 3, 2);
-    case BV_BASE: return SIFT_BLUR_FN(20, 1, 0);
-    case BV_LVL64: return SIFT_BLUR_FN(40, 0, 0);
-    default: return SIFT_BLUR_FN(40, 3, 0);
+    default: return SIFT_BLUR_FN(20, 1, 0);
   }
-#undef SIFT_BLUR_FN
 }
-// Radius R in 1 .. kMaxR.
-BlurFn blur_r1_4(int R, int variant);
-BlurFn blur_r5_8(int R, int variant);
-BlurFn blur_r9_12(int R, int variant);
-BlurFn blur_r13_16(int R, int variant);
+template <int R> BlurFn blur_instance64(int variant) {  // 40-row tiles
+  return variant == BV_LVL64 ? SIFT_BLUR_FN(40, 0, 0) : SIFT_BLUR_FN(40, 3, 0);
+}
+#undef SIFT_BLUR_FN
+// Of a radius in 1 .. kMaxR that blur_fn (pyramid.cu) does not instantiate itself.
+BlurFn blur_rest(int R, int variant);
+BlurFn blur_rest64(int R, int variant);
 
 }  // namespace sift

@@ -145,6 +145,16 @@ void Engine::set_taps() {
   }
 }
 
+cudaError_t Engine::load_blurs(bool rows64) {
+  if (rows64 && rows64_) return cudaSuccess;
+  unsigned radii = 0;
+  for (int R : base_R_) radii |= 1u << std::max(R, 0);
+  for (int l = 1; l <= S_ + 2; l++) radii |= 1u << lvl_R_[l];
+  const cudaError_t e = blur_set_attributes(radii, P_.fp16_pyramid != 0, rows64);
+  rows64_ = rows64 && e == cudaSuccess;
+  return e;
+}
+
 sift_status Engine::init() {
   if (inited_) return SIFT_OK;
   std::string why;
@@ -170,11 +180,8 @@ sift_status Engine::init() {
   }
   for (int o = 0; o < kMaxOct && e == cudaSuccess; o++)
     e = cudaEventCreateWithFlags(&fork_ev_[o], cudaEventDisableTiming);
-  unsigned radii = 0;
   set_taps();
-  for (int R : base_R_) radii |= 1u << std::max(R, 0);
-  for (int l = 1; l <= S_ + 2; l++) radii |= 1u << lvl_R_[l];
-  if (e == cudaSuccess) e = blur_set_attributes(radii);
+  if (e == cudaSuccess) e = load_blurs(false);
   if (e != cudaSuccess) {
     err = std::string("CUDA initialisation failed: ") + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? SIFT_E_OOM : SIFT_E_CUDA;
@@ -599,6 +606,16 @@ sift_status Engine::get_graph(int M, int modes, cudaGraphExec_t *out, bool pyram
     last_kernels_ = it->second.kernels;
     return SIFT_OK;
   }
+  // The larger row class is for tuned handles only: its kernels are loaded when a
+  // tuning first asks for them, before the capture.
+  bool rows64 = false;
+  for (int o = 0; o < M; o++)
+    for (int l = 1; l <= S_ + 2; l++) rows64 |= tun_.lvl_kind[o][l] == TK_BLUR64;
+  if (rows64 && load_blurs(true) != cudaSuccess) {
+    cudaGetLastError();
+    err = "blur kernels could not be loaded";
+    return SIFT_E_CUDA;
+  }
   GraphEntry ge;
   if (prof) ge.prof = new std::vector<ProfRec>();
   cudaError_t e = cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal);
@@ -851,6 +868,11 @@ sift_status Engine::autotune(int H, int W, cudaStream_t s) {
     cudaEventElapsedTime(&ms, a, b);
     return ms;
   };
+  if (st == SIFT_OK && load_blurs(true) != cudaSuccess) {
+    cudaGetLastError();
+    err = "blur kernels could not be loaded";
+    st = SIFT_E_CUDA;
+  }
   if (st == SIFT_OK) {
     for (int l = 0; l < kMaxLevels; l++) tun_.lvl_kind[0][l] = TK_BLUR32;
     float best = time_stage();

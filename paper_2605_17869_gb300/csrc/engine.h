@@ -156,6 +156,9 @@ class Engine {
 
  private:
   void set_taps();  // radii and taps of the base and level blurs
+  // Load the blur kernels of the handle's radii; rows64: also the larger row class.
+  cudaError_t load_blurs(bool rows64);
+  bool rows64_ = false;  // it is loaded
   sift_status fill_plan(int n, const ImgIn *imgs, Desc &hd, WsLayout &lay, int *max_oct) const;
   sift_status ensure_workspace(size_t bytes, cudaStream_t s);
   sift_status upload(Desc *hd, size_t bytes, cudaStream_t s);

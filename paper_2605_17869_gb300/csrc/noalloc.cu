@@ -95,7 +95,9 @@ cudaError_t setup_device(DeviceScratch &ds) {
   cudaError_t e = cudaGetSymbolAddress(&ptr, g_scratch);
   if (e == cudaSuccess) e = cudaGetSymbolAddress(&lb, g_lb);
   if (e == cudaSuccess) ds.lb = static_cast<unsigned long long *>(lb);
-  if (e == cudaSuccess) e = blur_set_attributes(~0u);  // every radius: later calls load no code
+  // Every radius, so that later calls load no code; the larger row class is for tuned
+  // handles only.
+  if (e == cudaSuccess) e = blur_set_attributes(~0u, true, false);
   if (e == cudaSuccess) e = descriptor_set_attributes();
   if (e == cudaSuccess) e = extrema_set_attributes();
   if (e == cudaSuccess && ptr) ds.ptr = ptr;

@@ -276,9 +276,22 @@ PolyTaps make_poly_taps(const BlurTaps &t, int R) {
 
 namespace {
 
+// The radii of three scales per octave at sigma0 1.6, the base blurs' among them, are
+// in this unit. A unit's code is loaded when the first of its kernels is asked for, which
+// takes some 0.4 ms and more the larger it is, and each kernel 6 us on top. With the
+// radii spread over four units of their own, a process's first sift_create took 3.7 ms
+// (three units) against 2.6 now, its first sift_extract_noalloc 4.0 against 3.35 (2.35
+// when one kernel with a runtime radius served the other radii).
 BlurFn blur_fn(int R, int variant) {
-  return R <= 4 ? blur_r1_4(R, variant) : R <= 8 ? blur_r5_8(R, variant)
-         : R <= 12 ? blur_r9_12(R, variant) : blur_r13_16(R, variant);
+  const bool rows64 = variant == BV_LVL64 || variant == BV_DEC64;
+  switch (R) {
+    case 5: return rows64 ? blur_instance64<5>(variant) : blur_instance<5>(variant);
+    case 7: return rows64 ? blur_instance64<7>(variant) : blur_instance<7>(variant);
+    case 8: return rows64 ? blur_instance64<8>(variant) : blur_instance<8>(variant);
+    case 10: return rows64 ? blur_instance64<10>(variant) : blur_instance<10>(variant);
+    case 13: return rows64 ? blur_instance64<13>(variant) : blur_instance<13>(variant);
+    default: return rows64 ? blur_rest64(R, variant) : blur_rest(R, variant);
+  }
 }
 
 int level_variant(int th_kind, bool m3, int storage) {
@@ -310,10 +323,12 @@ cudaError_t launch_fn(const BlurFn &f, int grid, cudaStream_t s, bool pdl, const
 
 int blur_tile_rows(int th_kind) { return tile_rows(th_kind); }
 
-cudaError_t blur_set_attributes(unsigned radii) {
+cudaError_t blur_set_attributes(unsigned radii, bool h16, bool rows64) {
   cudaError_t e = cudaSuccess;
   for (int R = 1; R <= kMaxR && e == cudaSuccess; R++)
     for (int v = (radii >> R & 1) ? 0 : BV_COUNT; v < BV_COUNT && e == cudaSuccess; v++) {
+      if (!h16 && (v == BV_LVL_H16 || v == BV_DEC_R16 || v == BV_DEC_H16)) continue;
+      if (!rows64 && (v == BV_LVL64 || v == BV_DEC64)) continue;
       const BlurFn f = blur_fn(R, v);
       e = cudaFuncSetAttribute(f.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem);
     }

@@ -228,8 +228,9 @@ cudaError_t launch_export(const Desc *d, float *out, int n_sm, cudaStream_t s);
 int blur_tile_rows(int th_kind);
 // mode: 0 level, 1 base as is, 2 magnified base, 3 level 1 from the previous octave.
 int blur_blocks_per_sm(int R, int th_kind, int mode, int storage = 0);
-// Allow the blur kernels of the radii in the mask (bit R) their shared memory.
-cudaError_t blur_set_attributes(unsigned radii);
+// Load the blur kernels of the radii in the mask (bit R) and allow them their shared
+// memory. h16: those of binary16 octaves too; rows64: those of the larger row class.
+cudaError_t blur_set_attributes(unsigned radii, bool h16, bool rows64);
 
 // Detection (detect.cu)
 // pdl: launch as a programmatic dependent of the previous kernel on s.
