@@ -568,7 +568,8 @@ constexpr int kDescWarpFloats = kDescLen * kDescCols;
 // 8 / 2 pi: the descriptors' distance from 64 bits is unchanged.
 __device__ __forceinline__ float atan2_eighths(float y, float x) {
   const float ax = fabsf(x), ay = fabsf(y);
-  const float t = fminf(ax, ay) * rcp_approx(fmaxf(fmaxf(ax, ay), 1.17549435e-38f));
+  // (no quotient of two infinities, and no reciprocal that is flushed to 0)
+  const float t = fminf(fminf(ax, ay), 0x1p126f) * rcp_approx(fminf(fmaxf(fmaxf(ax, ay), 1.17549435e-38f), 0x1p126f));
   const float u = t * t;
   float r = 0.00362859224f;
   r = fmaf(r, u, -0.0204592142f);
@@ -601,15 +602,16 @@ struct Vote {
   int cell;        // ((v0 * 4 + u0) * 8) * kDescCols, the first cell's histogram word
   bool ok[4];      // whether cells (v0, u0), (v0, u0 + 1), (v0 + 1, u0), (v0 + 1, u0 + 1) exist
   float w[4];      // spatial weights times the magnitude-Gaussian weight
-  int oe, oo;      // the even and the odd orientation bin, times kDescCols
-  float fe, fo;    // their orientation weights
+  int o[2];        // the orientation bins of the first and the second pass, times kDescCols
+  float f[2];      // their orientation weights
 };
 
 // ok false: the lane has no sample (its coordinates may lie anywhere); none of
 // its four cells exists, so that the commit skips it without a branch around
-// this function.
+// this function. upper: the lane is one of the upper half, whose first pass takes
+// the odd bin (the lower half's the even one).
 __device__ __forceinline__ void desc_targets(Vote &v, float rx, float ry, float gx, float gy,
-                                             float th8, bool ok = true) {
+                                             float th8, bool upper, bool ok = true) {
   const float u = rx + 1.5f, vv0 = ry + 1.5f;
   const float mag = sqrtf(gx * gx + gy * gy);
   float ob = atan2_eighths(gy, gx) - th8;
@@ -618,11 +620,13 @@ __device__ __forceinline__ void desc_targets(Vote &v, float rx, float ry, float 
   int u0, v0, o0;
   const float fu = u - split_floor(u, &u0), fv = vv0 - split_floor(vv0, &v0);
   const float f1 = ob - split_floor(ob, &o0);
-  const bool odd0 = o0 & 1;
-  v.oe = ((o0 + 1) & 6) * kDescCols;
-  v.oo = (o0 & 7 | 1) * kDescCols;
-  v.fe = odd0 ? f1 : 1.f - f1;
-  v.fo = 1.f - v.fe;
+  // Bin o0 has the weight 1 - f1, bin o0 + 1 the weight f1; one of them is even.
+  const int oe = ((o0 + 1) & 6) * kDescCols, oo = (o0 & 7 | 1) * kDescCols;
+  v.o[0] = upper ? oo : oe;
+  v.o[1] = upper ? oe : oo;
+  const bool lower_first = (o0 & 1) == (int)upper;
+  v.f[0] = lower_first ? 1.f - f1 : f1;
+  v.f[1] = lower_first ? f1 : 1.f - f1;
   v.cell = (v0 * 4 + u0) * (8 * kDescCols);
   const bool ua = (unsigned)u0 < 4u, ub = (unsigned)(u0 + 1) < 4u;
   const bool va = ok && (unsigned)v0 < 4u, vb = ok && (unsigned)(v0 + 1) < 4u;
@@ -630,11 +634,14 @@ __device__ __forceinline__ void desc_targets(Vote &v, float rx, float ry, float 
   v.ok[1] = va && ub;
   v.ok[2] = vb && ua;
   v.ok[3] = vb && ub;
-  const float w1 = wt * fv, w0 = wt - w1;
+  // Products of the fractions, not differences of the weights: where the magnitude
+  // overflows these would be NaN, and one NaN bin leaves the descriptor zero, while
+  // infinite bins take the clip value.
+  const float w1 = wt * fv, w0 = wt * (1.f - fv);
+  v.w[0] = w0 * (1.f - fu);
   v.w[1] = w0 * fu;
-  v.w[0] = w0 - v.w[1];
+  v.w[2] = w1 * (1.f - fu);
   v.w[3] = w1 * fu;
-  v.w[2] = w1 - v.w[3];
 }
 
 // Add the votes of the warp's lanes to the warp's columns in the two passes
@@ -644,12 +651,10 @@ __device__ __forceinline__ void desc_targets(Vote &v, float rx, float ry, float 
 __device__ __forceinline__ void desc_commit(float *hist, int lane, const Vote &v) {
   constexpr int kStep[4] = {0, 8 * kDescCols, 32 * kDescCols, 40 * kDescCols};
   float *col = hist + (lane & (kDescCols - 1)) + v.cell;
-  const bool upper = lane >= 16;
 #pragma unroll
   for (int pass = 0; pass < 2; pass++) {
-    const bool even = (pass == 0) != upper;
-    float *c = col + (even ? v.oe : v.oo);
-    const float f = even ? v.fe : v.fo;
+    float *c = col + v.o[pass];
+    const float f = v.f[pass];
     float h[4];
 #pragma unroll
     for (int k = 0; k < 4; k++) h[k] = v.ok[k] ? c[kStep[k]] : 0.f;
@@ -674,6 +679,7 @@ __device__ __forceinline__ void desc_sweep(const Desc *__restrict__ d, const Ref
   const int tid = threadIdx.x;
   const int pitch = od.pitch;
   const LevelView<HF> lv = level_at<HF>(L, lofs, pitch, r.x, r.y);
+  const bool upper = lane >= 16;
     if (!d->dsp) {
       // Samples: integer offsets (i, jy) in [-R, R]^2 inside the image whose
       // rotated bin coordinates fall in (-1, 4)^2, i.e. inside a square of half
@@ -765,9 +771,9 @@ __device__ __forceinline__ void desc_sweep(const Desc *__restrict__ d, const Ref
           const float ga = lv[oa + 1] - lv[oa - 1], ha = lv[oa + pitch] - lv[oa - pitch];
           const float gb = lv[ob + 1] - lv[ob - 1], hb = lv[ob + pitch] - lv[ob - pitch];
           Vote vt;
-          desc_targets(vt, rxa, rya, ga, ha, th8, oka);
+          desc_targets(vt, rxa, rya, ga, ha, th8, upper, oka);
           desc_commit(hist, lane, vt);
-          desc_targets(vt, rxb, ryb, gb, hb, th8, okb);
+          desc_targets(vt, rxb, ryb, gb, hb, th8, upper, okb);
           desc_commit(hist, lane, vt);
         }
         __syncwarp();  // the next round rewrites this warp's interval table
@@ -803,7 +809,7 @@ __device__ __forceinline__ void desc_sweep(const Desc *__restrict__ d, const Ref
                            fy * (gx1 * at(p2) + fx * at(p2 + 1));
           const float ym = gy1 * (gx1 * at(pm) + fx * at(pm + 1)) +
                            fy * (gx1 * at(p) + fx * at(p + 1));
-          desc_targets(vt, rx, ry, xp - xm, yp - ym, th8);
+          desc_targets(vt, rx, ry, xp - xm, yp - ym, th8, upper);
           desc_commit(hist, lane, vt);
         }
       }
