@@ -5,8 +5,8 @@
 // The DoG is never stored: every consumer recomputes D = G[i+1] - G[i] with the
 // same single FP32 subtraction, so all stages see identical values.
 //
-// Candidates are first marked in a bitmap (one warp ballot per 32 pixels and
-// layer), then compacted by a two-level prefix scan over bitmap words. The
+// Candidates are first marked in a bitmap (30 pixels of a row and layer per word,
+// by warp ballots), then compacted by a single-pass scan over bitmap words. The
 // bitmap's memory order is (octave, layer, row, column), so the candidate list
 // comes out in that canonical order independently of tile shapes or batch
 // composition.
@@ -185,8 +185,8 @@ __device__ __forceinline__ void ext_test(const ExtRow<S> &P, const ExtRow<S> &C,
 // not depend on the tiling. Bitmap words are written by ballots; no atomics.
 // Two columns per lane share the copies, the loop, two of four shuffles per layer
 // and the middle values of the three-column extrema. What bounds the scan is the
-// ALU pipe (66%: three-input extrema and comparisons) together with HBM (52%, every
-// level value read once) at 16 warps per SM, which 128 registers allow (12 warps at
+// ALU pipe (64%: three-input extrema and comparisons) together with HBM (62%, 73% of
+// the measured copy; every level value read once) at 16 warps per SM, which 128 registers allow (12 warps at
 // 150: 2 percent more per call on the 64-image batch); rings of 4 and 8 rows were no
 // faster than 3. All scans of the 64-image batch: 545 us with one column per lane
 // (4.9 warp instructions per pixel and warp row), 480 with two (3.5), 439 with the

@@ -79,8 +79,8 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long *m, unsigned pa
       : "memory");
   return ok != 0;
 }
-// Bounded: gives up after kMaxPolls polls (each may suspend the thread briefly),
-// another thread of the block has, which *abort records.
+// Bounded: false after kMaxPolls polls (each may suspend the thread briefly), or once
+// another thread of the block has given up, which *abort records.
 __device__ __forceinline__ bool mbar_wait(unsigned long long *m, unsigned parity, volatile int *abort) {
   for (unsigned i = 0; i < kMaxPolls; i++) {
     if (mbar_try_wait(m, parity)) return true;

@@ -1,8 +1,6 @@
 // Gaussian scale space (§3.2, "GPU Pipeline Stages"): the launches of the level
 // blurs (blur.cuh), the 2x magnified first octave (k_base_poly, a polyphase
 // filter of the input, below) and the pyramid export.
-#include <type_traits>
-
 #include "blur.cuh"
 
 namespace sift {
@@ -144,13 +142,13 @@ struct PolyTaps {
   float c[2][2 * kPolyMaxQ + 1];
 };
 
-struct TileGeo {
+struct PolyTile {
   const float *src;
   float *out;
   int spitch, pitch, H, W, sh, sw, x0, y0;
 };
-__device__ __forceinline__ TileGeo tile_geo(const Desc *__restrict__ d, const int *pre, int t) {
-  TileGeo g;
+__device__ __forceinline__ PolyTile poly_tile(const Desc *__restrict__ d, const int *pre, int t) {
+  PolyTile g;
   const int b = find_owner(pre, d->n_img, t);
   const OctDev od = d->oct[b * kMaxOct];
   const ImgDev &im = d->img[b];
@@ -180,7 +178,7 @@ __global__ void __launch_bounds__(kPolyThreads) k_base_poly(const Desc *__restri
   const int G = gridDim.x;
   for (int t = blockIdx.x; t < total; t += G) {
     if (t + G >= total) pdl_trigger();  // successors launch during this block's last tile
-    const TileGeo g = tile_geo(d, pre, t);
+    const PolyTile g = poly_tile(d, pre, t);
     const int kx0 = g.x0 >> 1, ky0 = g.y0 >> 1;
     const int iyb = ky0 - Q, ixb = kx0 - Q;
     if (iyb >= 0 && iyb + NR <= g.sh && ixb >= 0 && ixb + NC <= g.sw) {
