@@ -68,7 +68,9 @@ typedef enum {
 typedef struct {
   int n_scales;          /* S: scales per octave (2..6) */
   float sigma0;          /* base scale of each octave; > 0 */
-  float init_blur;       /* blur already present in the input; >= 0 */
+  float init_blur;       /* blur already present in the input; >= 0. From sigma0
+                            (sigma0 / 2 for a magnified input) upwards level 0
+                            is the input (its magnification) as it is */
   int upsample;          /* 1: first octave from the 2x bilinear magnified input */
   int min_octave_side;   /* keep octaves while min(H_o, W_o) >= this; >= 16,
                             above the largest blur radius and 2 x border */
