@@ -56,7 +56,7 @@ void lookback_config(int *spins, int *hold);
 // Part of every tuning-cache key, raised whenever the kernels that were timed or
 // what a tuning's numbers mean change, so that a cache file's earlier entries are
 // not applied (they would be shapes that nothing measured). 2: row classes 32 and 64
-// are tiles of 20 and 40 rows; entries without a number were tuned for 32 and 64 rows.
+// are tiles of 20 and 40 rows; entries without a number may be for tiles of 32 and 64.
 constexpr int kTuningKernels = 2;
 Tuning default_tuning();
 std::string tuning_json(const Tuning &t, int n_scales);
